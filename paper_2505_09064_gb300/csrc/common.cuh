@@ -340,8 +340,48 @@ __host__ __device__ inline long long block_index(int q, long long k, long long n
 // A dropped pivot (drop[j] != 0) removes direction j: y_j is set to 0 in both
 // passes.  Used by the coarsest-level solves of the V-cycle and of
 // vasmg_coarse_solve_noalloc.
+// Up to 32 unknowns (every level coarsened to the root: 8 or 24) stay in the
+// lanes' registers, the factor's entries in flight eight steps ahead, and each
+// division is a product with the reciprocal (taken once, all pivots at the same
+// time) corrected by its residual: a step is four dependent FP64 operations
+// and a shuffle instead of a division and a round trip through memory.
 __device__ __forceinline__ void chol_substitute_warp(const double* chol, const uint8_t* drop, int n, double* y) {
   const int lane = threadIdx.x & 31;
+  if (n <= 32) {
+    constexpr unsigned FULL = 0xffffffffu;
+    const bool in = lane < n;
+    double v = in ? y[lane] : 0.0;
+    const double piv = in && !drop[lane] ? chol[(long long)lane * n + lane] : 0.0;
+    const double inv = piv != 0.0 ? 1.0 / piv : 0.0;
+    for (int pass = 0; pass < 2; ++pass) {
+      for (int t0 = 0; t0 < n; t0 += 8) {
+        double c[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const int j = pass == 0 ? t0 + u : n - 1 - (t0 + u);
+          c[u] = 0.0;
+          if (in && t0 + u < n) {
+            if (pass == 0 && lane > j) c[u] = chol[(long long)lane * n + j];
+            if (pass == 1 && lane < j) c[u] = chol[(long long)j * n + lane];
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          if (t0 + u < n) {
+            const int j = pass == 0 ? t0 + u : n - 1 - (t0 + u);
+            double q = v * inv;
+            q = fma(fma(-piv, q, v), inv, q);
+            const double yj = __shfl_sync(FULL, q, j);
+            v = lane == j ? yj : fma(-c[u], yj, v);
+          }
+        }
+      }
+    }
+    __syncwarp();
+    if (in) y[lane] = v;
+    __syncwarp();
+    return;
+  }
   for (int j = 0; j < n; ++j) {
     const double ljj = chol[(long long)j * n + j];
     const double yj = drop[j] ? 0.0 : y[j] / ljj;

@@ -334,6 +334,7 @@ struct Engine : EngineBase {
   // gamma-cycle (gamma >= 2): each level's coarse right-hand side and first
   // coarse correction, kept while the next coarse cycle runs
   std::vector<DevBuf<V>> wb, we;
+  std::vector<DevBuf<V>> xg;  // tail levels kept in shared memory: the prolongation's copy of x
   // 3D region levels: the sweeps' operator parts in the staged order
   // (vstaged_kernel), [0] the forward sweep's lower part, [1] the backward
   // sweep's whole rows, each built for the level's lanes per row G
@@ -645,7 +646,7 @@ struct Engine : EngineBase {
       i64 work = 0;
       for (int l = lt; l < L; ++l) work += c->S[l].nnz;
       nct = 1;
-      while (nct < 16 && work > (i64)nct * 4 * TAIL_THREADS * 8) nct *= 2;
+      while (nct < 16 && work > (i64)nct * 4096) nct *= 2;
       if (nct > 8)
         if (cudaFuncSetAttribute(tail_kernel<D, V, S>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
             cudaSuccess)
@@ -654,7 +655,7 @@ struct Engine : EngineBase {
       while (nct > 1) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(nct);
-        cfg.blockDim = dim3(TAIL_THREADS);
+        cfg.blockDim = dim3(tail_threads<D, V>());
         cudaLaunchAttribute at[1];
         at[0].id = cudaLaunchAttributeClusterDimension;
         at[0].val.clusterDim.x = nct;
@@ -668,6 +669,12 @@ struct Engine : EngineBase {
         cudaGetLastError();
         nct /= 2;
       }
+    }
+    // the prolongation's copies of the tail levels' x (see layout_tail)
+    xg.resize(L);
+    for (int l = lt; l < L; ++l) {
+      const size_t need = (size_t)c->S[l].nv * xs_bytes<D, V>();
+      if (need <= (size_t)TAIL_SMEM_MAX) xg[l].alloc((i64)((need + 15) / 16 * 16 / sizeof(V)), s);
     }
     // coarsest
     coarse_y.alloc(c->nc, s);
@@ -1044,19 +1051,20 @@ struct Engine : EngineBase {
   // First level of the one-CTA part of a tail that starts at level l0.
   int one_cta_start(int l0) const {
     int ls = L - 1;
-    while (ls > l0 && c->S[ls - 1].nv <= ONE_CTA_NV) --ls;
+    while (ls > l0 && c->S[ls - 1].nv <= one_cta_nv<V>()) --ls;
     return ls;
   }
-  // The tail's level tables; levels ls..L-1 get shared-memory slots.
-  // Returns the dynamic shared memory in bytes.
-  size_t fill_tail_args(TailArgs<V>& ta, int l0, int ls) {
+  // The tail's level tables; levels ls..L-1 get shared-memory slots when one
+  // CTA runs them.  Returns the dynamic shared memory in bytes.
+  size_t fill_tail_args(TailArgs<V>& ta, int l0, int ls, bool one_cta = true) {
     std::memset(&ta, 0, sizeof(ta));
     ta.l0 = l0;
     ta.L = L - 1;
     ta.ls = ls;
     ta.kd = -1;
+    ta.abort = sc.get() ? &sc.get()->abort : nullptr;
     size_t smem = 0;
-    for (int l = ta.ls; l < L; ++l) {
+    for (int l = ta.ls; l < L && one_cta; ++l) {
       ta.soff[l] = (int)(smem / sizeof(V));
       smem += 3 * sizeof(V) * (size_t)c->S[l].nv * D;
       smem = (smem + 15) / 16 * 16;
@@ -1087,8 +1095,37 @@ struct Engine : EngineBase {
       t.rw = v.rw;
       t.bc = v.bc;
       t.xc = v.xc;
+      t.xoff = -1;
     }
     ta.co = co;
+    return smem;
+  }
+  // The arguments of a tail launch from level l0: the dense level if there is
+  // one, else the one-CTA levels, and above them the levels whose x the CTAs
+  // keep in shared memory (the smaller ones first).  *base: the shared memory
+  // before the staging of b_kd; returns all of it.
+  size_t layout_tail(TailArgs<V>& ta, int l0, size_t* base) {
+    const bool dense = kd >= 0 && kd >= l0;
+    size_t smem = fill_tail_args(ta, l0, dense ? kd : one_cta_start(l0), !dense);
+    *base = smem;
+    if (dense) {
+      ta.kd = kd;
+      ta.dn = dn;
+      ta.dld = dld;
+      ta.dm = dm.get();
+      ta.dsoff = (int)(smem / sizeof(V));  // fill_tail_args keeps smem a multiple of 16 bytes
+      smem += sizeof(V) * (size_t)dld;
+    }
+    smem = (smem + 15) / 16 * 16;
+    for (int l = ta.ls - 1; l >= l0; --l) {
+      const size_t need = (size_t)c->S[l].nv * xs_bytes<D, V>();
+      if (c->S[l].ncol > TAIL_MAX_COLOURS || smem + need > (size_t)TAIL_SMEM_MAX) continue;
+      ta.lv[l].xoff = (int)(smem / sizeof(V));
+      ta.lv[l].xg = xg[l].get();
+      ta.nbar = std::max(ta.nbar, (int)c->S[l].ncol);
+      smem = (smem + need + 15) / 16 * 16;
+    }
+    VASMG_CHECK(smem <= (size_t)TAIL_SMEM_MAX, VASMG_ERR_UNSUPPORTED, "tail levels too large for shared memory");
     return smem;
   }
   // The V-cycle from the dense level kd down, as the matrix M (one CTA per
@@ -1117,8 +1154,7 @@ struct Engine : EngineBase {
     // level with per-level launches instead
     if (!c->dense_coarse || c->gamma >= 2) return;
     if constexpr (std::is_same<V, float>::value) {
-      const int ls = one_cta_start(lt);
-      for (int l = ls; l < L; ++l) {
+      for (int l = one_cta_start(lt); l < L; ++l) {
         const i64 n = c->S[l].nv * D;
         if (n * n <= (i64)nct * DENSE_ROWS_PER_CTA * DENSE_ROWS_PER_CTA) {
           kd = l;
@@ -1129,16 +1165,6 @@ struct Engine : EngineBase {
       cudaStream_t s = c->stream;
       dn = (int)(c->S[kd].nv * D);
       dld = (dn + 3) / 4 * 4;
-      {
-        // the tail stages b_kd in shared memory beside its levels' vectors
-        TailArgs<V> probe;
-        const size_t need = fill_tail_args(probe, lt, ls) + sizeof(V) * (size_t)dld;
-        if (need > (size_t)TAIL_SMEM_MAX) {
-          kd = -1;
-          dn = 0;
-          return;
-        }
-      }
       if (dm.n != (i64)dn * dld) dm.alloc((i64)dn * dld, s);
       dm.zero();
       DevBuf<double> ys;
@@ -1147,25 +1173,17 @@ struct Engine : EngineBase {
       const size_t smem = fill_tail_args(ta, kd, kd);
       ta.dn = dn;
       ta.dld = dld;
-      dense_level_kernel<D, V, S><<<dn, TAIL_THREADS, smem, s>>>(ta, dm.get(), ys.get());
+      dense_level_kernel<D, V, S><<<dn, tail_threads<D, V>(), smem, s>>>(ta, dm.get(), ys.get());
       check_launch("dense_level");
     }
   }
   void tail(int l0, cudaStream_t s) {
     TailArgs<V> ta;
-    size_t smem = fill_tail_args(ta, l0, one_cta_start(l0));
-    if (kd >= 0 && kd >= ta.ls) {
-      ta.kd = kd;
-      ta.dn = dn;
-      ta.dld = dld;
-      ta.dm = dm.get();
-      ta.dsoff = (int)(smem / sizeof(V));  // fill_tail_args keeps smem a multiple of 16 bytes
-      smem += sizeof(V) * (size_t)dld;
-      VASMG_CHECK(smem <= (size_t)TAIL_SMEM_MAX, VASMG_ERR_UNSUPPORTED, "tail levels too large for shared memory");
-    }
+    size_t base = 0;
+    const size_t smem = layout_tail(ta, l0, &base);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(nct);
-    cfg.blockDim = dim3(TAIL_THREADS);
+    cfg.blockDim = dim3(tail_threads<D, V>());
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute at[1];
@@ -1427,14 +1445,7 @@ struct Engine : EngineBase {
       v.nv.push_back(c->S[l].nv);
       v.pnnz.push_back(l + 1 < L ? (double)c->C[l].pnnz : 0.0);
     }
-    v.tail_smem = fill_tail_args(v.ta, lt, one_cta_start(lt));
-    if (kd >= 0 && kd >= v.ta.ls) {
-      v.ta.kd = kd;
-      v.ta.dn = dn;
-      v.ta.dld = dld;
-      v.ta.dm = dm.get();
-      v.ta.dsoff = (int)(v.tail_smem / sizeof(V));
-    }
+    v.tail_smem = layout_tail(v.ta, lt, &v.tail_smem_base);
     v.cga = cga;
     v.cga.cond = 0;
     v.cg_blocks = cg_blocks;

@@ -13,12 +13,24 @@
 namespace vasmg {
 
 constexpr int TAIL_NV = 20000;
-constexpr int TAIL_THREADS = 1024;
-constexpr int TAIL_G = 8;
-// lanes per row in the tail: 3D coarse rows hold ~100 blocks
+// Threads of a tail CTA.  A lane keeps the entries of its next two rows in
+// registers (tail_sweep): up to 128 registers a thread in 2D FP32, 168 in 2D
+// FP64, 255 in 3D.
+template <int D, typename V>
+constexpr int tail_threads() { return D == 3 ? 256 : (sizeof(V) == 8 ? 384 : 512); }
+constexpr int TAILB_THREADS = 256;  // the batched tail: 2D and 3D hierarchies in one launch
+// Lanes per row in the tail: 3D coarse rows hold ~100 blocks.
 template <int D>
-constexpr int tail_g() { return D == 2 ? TAIL_G : 32; }
-constexpr int ONE_CTA_NV = 1200;  // tail levels this small run on one CTA
+constexpr int tail_g() { return D == 2 ? 8 : 32; }
+// Entries per lane loaded ahead of a colour's barrier: whole rows of the usual
+// length (24 blocks in 2D, 100 to 125 in 3D), as far as the registers go.
+template <int D, typename V>
+constexpr int tail_npf() { return D == 2 ? 3 : (sizeof(V) == 8 ? 3 : 4); }
+// Tail levels this small run on one CTA, their vectors in shared memory.  An
+// FP64 level is bound by one SM's FP64 rate there (3D, 729 vertices: ~500 us per
+// V-cycle), so only the smallest stay on one CTA.
+template <typename V>
+constexpr int one_cta_nv() { return sizeof(V) == 8 ? 100 : 1200; }
 // Dynamic shared memory the tail kernel is configured for.  The limit is an
 // attribute of the kernel function, shared by every handle in the process, so
 // every engine sets the same value once instead of its own size: a handle
@@ -335,34 +347,6 @@ __device__ __forceinline__ void row_entries(const L_t& L, const RowSeg& sg, int 
   }
 }
 
-// One row of a sweep / residual by a group of G lanes.
-// MODE 0: x_i = Dinv (b_i - lower part), MODE 1: x_i = Dinv (b_i - all
-// off-diagonal blocks), MODE 2: r_i = -(upper part).
-template <int D, int G, typename V, typename S, int MODE, typename L_t, bool LC = false>
-__device__ __forceinline__ void row_pass(const L_t& L, int row, bool valid, int lane) {
-  RowSeg sg{0, 0, 0, 0};
-  if (valid) sg = seg_range<MODE>(L, row);
-  V acc[D];
-#pragma unroll
-  for (int a = 0; a < D; ++a) acc[a] = V(0);
-  row_entries<D, G, V, S, MODE, LC, true>(L, sg, lane, acc);
-#pragma unroll
-  for (int o = G / 2; o > 0; o >>= 1)
-#pragma unroll
-    for (int a = 0; a < D; ++a) acc[a] += __shfl_xor_sync(0xffffffffu, acc[a], o, G);
-  if (!valid || lane >= D) return;
-  if (MODE == 2) {
-    stx<LC>(L.r + (long long)row * D + lane, -pick<D>(acc, lane));
-  } else {
-    V s = V(0);
-#pragma unroll
-    for (int bb = 0; bb < D; ++bb)
-      s += __ldg((const V*)L.dinv + (long long)(lane * D + bb) * L.nv + row) *
-           (ldx<LC>((const V*)L.b + (long long)row * D + bb) - acc[bb]);
-    stx<LC>(L.x + (long long)row * D + lane, s);
-  }
-}
-
 // Entries a lane keeps in registers between the prefetch and the finish of a row.
 template <int D, typename V, int NPF_ = ((D * D * sizeof(V) <= 16) ? 2 : 1)>
 struct RowPF {
@@ -470,6 +454,49 @@ __device__ __forceinline__ void restrict_row(const L_t& L, int I) {
   }
 #pragma unroll
   for (int a = 0; a < D; ++a) stx<LC>((V*)L.bc + (long long)I * D + a, acc[a]);
+}
+
+// The same sum for the 4 lanes of a group: each lane fetches one entry in four
+// (all of them in flight), and every lane adds all of them in entry order.
+template <int D, typename V, typename L_t>
+__device__ __forceinline__ void restrict_row_g4(const L_t& L, int I, bool valid, int lane) {
+  constexpr unsigned FULL = 0xffffffffu;
+  constexpr int U = 8;  // entries per lane fetched together
+  V acc[D];
+#pragma unroll
+  for (int a = 0; a < D; ++a) acc[a] = V(0);
+  const int t0 = valid ? __ldg(L.rrp + I) : 0, t1 = valid ? __ldg(L.rrp + I + 1) : 0;
+  for (int t = t0; __any_sync(FULL, t < t1); t += 4 * U) {
+    V w[U], r[U][D];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int e = t + 4 * u + lane;
+      w[u] = V(0);
+#pragma unroll
+      for (int a = 0; a < D; ++a) r[u][a] = V(0);
+      if (e < t1) {
+        w[u] = __ldg((const V*)L.rw + e);
+        ldx_vertex<D, false, true, false>((const V*)L.r + (long long)__ldg(L.rci + e) * D, r[u]);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int n = t1 - (t + 4 * u);  // entries of this fetch
+      if (!__any_sync(FULL, n > 0)) break;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const V wq = __shfl_sync(FULL, w[u], q, 4);
+#pragma unroll
+        for (int a = 0; a < D; ++a) {
+          const V rq = __shfl_sync(FULL, r[u][a], q, 4);
+          if (q < n) acc[a] += wq * rq;
+        }
+      }
+    }
+  }
+  if (valid && lane == 0)
+#pragma unroll
+    for (int a = 0; a < D; ++a) stx<false>((V*)L.bc + (long long)I * D + a, acc[a]);
 }
 
 template <int D, typename V, typename L_t, bool LC = false>
@@ -823,6 +850,7 @@ __device__ __forceinline__ bool mbar_test(unsigned long long* b, unsigned parity
 // flag, or soon after another wait raised it (read every 256 polls; never
 // when abort_flag is null).
 __device__ __forceinline__ bool mbar_wait(unsigned long long* b, unsigned parity, int* abort_flag) {
+#pragma unroll 1
   for (int spins = 0;; ++spins) {
     if (mbar_test(b, parity)) return true;
     if (spins >= SPIN_LIMIT) {
@@ -1164,6 +1192,8 @@ struct TL {
   const V* rw;
   V* bc;
   const V* xc;
+  int xoff;  // shared-memory offset (in V) of the level's x in every CTA of the cluster, or -1
+  V* xg;     // the same copy in global memory, written by the prolongation
 };
 
 // A tail level keeps the combined CSR: one segment, [rp, sp) lower, [sp,
@@ -1190,10 +1220,12 @@ template <typename V>
 struct TailArgs {
   int l0, L;                     // levels l0..L handled here, L = coarsest
   int ls;                        // levels ls..L run on CTA 0 alone
-  int kd;                        // dense level (ls <= kd <= L) or -1: x_kd = M b_kd replaces levels kd..L
+  int kd;                        // dense level (= ls) or -1: x_kd = M b_kd replaces levels kd..L
   int dn;                        // n_kd = nv_kd * d, the order of M
   int dld;                       // row stride of M: dn rounded up to a multiple of 4 (zero padding)
   int dsoff;                     // shared-memory offset (in V, 16-byte aligned) of b_kd staged for M b_kd
+  int nbar;                      // most colours of a level with its x in shared memory
+  int* abort;                    // raised by a wait that gave up
   const V* dm;                   // M, row-major dn x dld: the V-cycle from level kd as a matrix
   int soff[MAX_LEVELS];          // shared-memory offset (in V) of x_l, b_l, r_l for l >= ls
   TL<V> lv[MAX_LEVELS];
@@ -1215,45 +1247,413 @@ __device__ __forceinline__ unsigned cluster_size() {
   return r;
 }
 
-struct ClusterSync {
-  __device__ __forceinline__ void operator()() const { cluster_sync_all(); }
+// A d x d block in registers as it is stored: BF16 stays packed.
+template <int D, typename V, typename S>
+struct BlkReg {
+  V a[D * D];
+  __device__ __forceinline__ void load(const S* op, long long n, int k) {
+    if constexpr (D == 2) {
+      (void)n;
+      ldv4<V, S>(op + (long long)k * 4, a);
+    } else {
+      ldv8<V, S>(op + (long long)k * 8, a);
+      a[8] = ldv<V, S>(op + 8 * n + k);
+    }
+  }
+  __device__ __forceinline__ V at(int q) const { return a[q]; }
 };
-struct CtaSync {
-  __device__ __forceinline__ void operator()() const { __syncthreads(); }
+template <int D>
+struct BlkReg<D, float, __nv_bfloat16> {
+  unsigned w[D == 2 ? 2 : 5];
+  __device__ __forceinline__ void load(const __nv_bfloat16* op, long long n, int k) {
+    if constexpr (D == 2) {
+      (void)n;
+      const uint2 t = __ldg(reinterpret_cast<const uint2*>(op + (long long)k * 4));
+      w[0] = t.x, w[1] = t.y;
+    } else {
+      const uint4 t = __ldg(reinterpret_cast<const uint4*>(op + (long long)k * 8));
+      w[0] = t.x, w[1] = t.y, w[2] = t.z, w[3] = t.w;
+      w[4] = __ldg(reinterpret_cast<const unsigned short*>(op + 8 * n + k));
+    }
+  }
+  __device__ __forceinline__ float at(int q) const {
+    return __uint_as_float((q & 1) ? (w[q >> 1] & 0xffff0000u) : (w[q >> 1] << 16));
+  }
+};
+
+// Where a tail level's x lives during its sweeps.
+//  X_GLOBAL  global memory, phases separated by cluster barriers (a level too
+//            large for the CTAs' shared memory);
+//  X_CTA     one CTA's shared memory, phases separated by CTA barriers;
+//  X_CLUSTER a copy in the shared memory of every CTA of the cluster.  A row's
+//            values go to all the copies with st.async, which counts its bytes
+//            on the receiver's mbarrier of the row's colour; a CTA starts a
+//            colour when its barrier of the colour before has all the bytes.  A
+//            step then needs no release to L2 and no cluster barrier, and
+//            gathers from its own shared memory.
+enum { X_GLOBAL = 0, X_CTA = 1, X_CLUSTER = 2 };
+
+// values of x per vertex of an X_CLUSTER copy (3D FP32: one 16-byte store)
+template <int D, typename V>
+constexpr int xs_stride() { return (D == 3 && sizeof(V) == 4) ? 4 : D; }
+template <int D, typename V>
+constexpr int xs_bytes() { return xs_stride<D, V>() * (int)sizeof(V); }
+
+template <int D, typename V>
+__device__ __forceinline__ void xs_gather(const V* xs, int j, V (&v)[D]) {
+  const V* p = xs + j * xs_stride<D, V>();
+  if constexpr (D == 2 && sizeof(V) == 4) {
+    const float2 t = *reinterpret_cast<const float2*>(p);
+    v[0] = t.x, v[1] = t.y;
+  } else if constexpr (D == 2) {
+    const double2 t = *reinterpret_cast<const double2*>(p);
+    v[0] = t.x, v[1] = t.y;
+  } else if constexpr (sizeof(V) == 4) {
+    const float4 t = *reinterpret_cast<const float4*>(p);
+    v[0] = t.x, v[1] = t.y, v[2] = t.z;
+  } else {
+    v[0] = p[0], v[1] = p[1], v[2] = p[2];
+  }
+}
+
+__device__ __forceinline__ unsigned cluster_addr(unsigned a, unsigned rank) {
+  unsigned r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+  return r;
+}
+// x of one vertex to CTA `rank`'s copy (a, bar: this CTA's addresses of the
+// entry and of the mbarrier that counts it)
+template <int D, typename V>
+__device__ __forceinline__ void xs_send(unsigned a, unsigned bar, unsigned rank, const V (&v)[D]) {
+  const unsigned ra = cluster_addr(a, rank), rb = cluster_addr(bar, rank);
+  if constexpr (D == 2 && sizeof(V) == 4) {
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%1, %2}, [%3];" ::"r"(ra),
+                 "r"(__float_as_uint(v[0])), "r"(__float_as_uint(v[1])), "r"(rb));
+  } else if constexpr (sizeof(V) == 4) {
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(
+                     ra),
+                 "r"(__float_as_uint(v[0])), "r"(__float_as_uint(v[1])), "r"(__float_as_uint(v[2])), "r"(0u), "r"(rb));
+  } else {
+#pragma unroll
+    for (int a8 = 0; a8 < D; ++a8)
+      asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(ra + 8 * a8),
+                   "l"(__double_as_longlong(v[a8])), "r"(rb));
+  }
+}
+// The sum over a group of G lanes of each component, component own_comp(lane)
+// in each lane: half the lanes pass on half of the components at the first
+// steps (a quarter of the shuffles and additions of D butterflies, which FP64
+// runs at ~60 clocks each per SM partition); every component's sum has the
+// additions of its butterfly.
+template <int D, int G>
+__device__ __forceinline__ int own_comp(int lane) {
+  return D == 2 ? ((lane & (G / 2)) ? 1 : 0) : ((lane & (G / 2)) ? 2 : 0) + ((lane & (G / 4)) ? 1 : 0);
+}
+template <int D, int G>
+constexpr int own_step() { return D == 2 ? G / 2 : G / 4; }  // component a: lanes a own_step .. (a + 1) own_step - 1
+template <int D, int G, typename V>
+__device__ __forceinline__ V group_sum_own(const V (&acc)[D], int lane) {
+  constexpr unsigned FULL = 0xffffffffu;
+  const bool hi = lane & (G / 2);
+  V r;
+  if constexpr (D == 2) {
+    r = (hi ? acc[1] : acc[0]) + __shfl_xor_sync(FULL, hi ? acc[0] : acc[1], G / 2, G);
+  } else {
+    const V a = (hi ? acc[2] : acc[0]) + __shfl_xor_sync(FULL, hi ? acc[0] : acc[2], G / 2, G);
+    const V b = (hi ? V(0) : acc[1]) + __shfl_xor_sync(FULL, hi ? acc[1] : V(0), G / 2, G);
+    const bool q = lane & (G / 4);
+    r = (q ? b : a) + __shfl_xor_sync(FULL, q ? a : b, G / 4, G);
+  }
+#pragma unroll
+  for (int o = own_step<D, G>() / 2; o > 0; o >>= 1) r += __shfl_xor_sync(FULL, r, o, G);
+  return r;
+}
+
+// A tail row as one lane of its group holds it ahead of its colour: its first
+// NPF entries and (sweeps) its component's row of the diagonal inverse and b.
+template <int D, typename V, typename S, int NPF>
+struct TailRow {
+  int a0, len;
+  int col[NPF];
+  BlkReg<D, V, S> blk[NPF];
+  V di[D], bv;
+};
+
+template <int D, int G, typename V, typename S, int MODE, bool LC, int NPF>
+__device__ __forceinline__ void tail_row_load(const TL<V>& L, int row, bool valid, int lane, const RowSeg& sg,
+                                              TailRow<D, V, S, NPF>& st) {
+  st.a0 = sg.a0;
+  st.len = sg.len;
+#pragma unroll
+  for (int p = 0; p < NPF; ++p) {
+    const int e = lane + p * G;
+    st.col[p] = -1;
+    if (e < sg.len) {
+      st.col[p] = __ldg(L.ci + sg.a0 + e);
+      st.blk[p].load((const S*)L.off, L.nnz, sg.a0 + e);
+    }
+  }
+  const int own = own_comp<D, G>(lane);
+  if (MODE != 2 && valid && own < D) {
+#pragma unroll
+    for (int bb = 0; bb < D; ++bb) st.di[bb] = __ldg((const V*)L.dinv + (long long)(own * D + bb) * L.nv + row);
+    st.bv = ldx<LC>((const V*)L.b + (long long)row * D + own);
+  }
+}
+
+// The row's gathers of x, all in flight together, and its sum in the order of
+// row_pass.  Returns component own_comp(lane) of x (MODE 0, 1) or r (MODE 2).
+template <int D, int G, typename V, typename S, int MODE, int XM, int NPF>
+__device__ __forceinline__ V tail_row_value(const TL<V>& L, const V* xs, int lane, const TailRow<D, V, S, NPF>& st) {
+  constexpr bool LC = XM == X_CTA;
+  auto gather = [&](int j, V(&v)[D]) {
+    if constexpr (XM == X_CLUSTER) xs_gather<D, V>(xs, j, v);
+    else ldx_vertex<D, LC, false, false>((const V*)L.x + (long long)j * D, v);
+  };
+  V xj[NPF][D];  // (every slot gathers, entry or not: registers left as they were would stay live around every loop)
+#pragma unroll
+  for (int p = 0; p < NPF; ++p) gather(max(st.col[p], 0), xj[p]);
+  V acc[D];
+#pragma unroll
+  for (int a = 0; a < D; ++a) acc[a] = V(0);
+#pragma unroll
+  for (int p = 0; p < NPF; ++p) {
+    if (st.col[p] >= 0) {
+#pragma unroll
+      for (int a = 0; a < D; ++a)
+#pragma unroll
+        for (int bb = 0; bb < D; ++bb) acc[a] += st.blk[p].at(a * D + bb) * xj[p][bb];
+    }
+  }
+#pragma unroll 1
+  for (int e = lane + NPF * G; e < st.len; e += G) {
+    BlkReg<D, V, S> blk;
+    const int j = __ldg(L.ci + st.a0 + e);
+    blk.load((const S*)L.off, L.nnz, st.a0 + e);
+    V x[D];
+    gather(j, x);
+#pragma unroll
+    for (int a = 0; a < D; ++a)
+#pragma unroll
+      for (int bb = 0; bb < D; ++bb) acc[a] += blk.at(a * D + bb) * x[bb];
+  }
+  const V sum = group_sum_own<D, G>(acc, lane);
+  if (MODE == 2) return -sum;
+  const V t = st.bv - sum;
+  V v = V(0);
+#pragma unroll
+  for (int bb = 0; bb < D; ++bb) v += st.di[bb] * __shfl_sync(0xffffffffu, t, bb * own_step<D, G>(), G);
+  return v;
+}
+
+// Shared memory of the mbarriers that count the bytes of an X_CLUSTER sweep's
+// colours.  Each sweep completes one phase of all of the first `nbar`: the
+// colours' with their rows' bytes, the others at once.
+constexpr int TAIL_MAX_COLOURS = 512;
+struct XBars {
+  unsigned long long* bar;
+  unsigned parity;  // of the phase the current sweep completes
+  int nbar, nct;
+  int* abort;
+  int* cs;          // shared memory for the level's colour starts (the row after next's address waits for them)
 };
 
 // One multicolour sweep of a tail level (MODE 0: forward from zero, MODE 1:
-// backward), colours separated by `sync`.  Group gg of NG handles rows
-// base + gg; the entries, diagonal inverse and b of the next pass (the next
-// colour's first pass at the end of a colour) are loaded before the barrier,
-// since no phase of the sweep writes them; only the x gather follows it.
-template <int D, int G, typename V, typename S, int MODE, bool LC, typename Sync>
-__device__ __forceinline__ void tail_sweep(const TL<V>& L, int gg, int NG, int lane, Sync sync) {
+// backward).  Group gg of NG handles rows base + gg.  Ahead of a colour each
+// lane has loaded its entries of the group's next two rows (an L2 round trip
+// takes about as long as a colour's step), and the range of the one after them,
+// so what follows the colour's barrier is the gathers of x, one shuffle sum and
+// the store.  `out`: x is also written to global memory.
+template <int D, int G, typename V, typename S, int MODE, int XM>
+__device__ __forceinline__ void tail_sweep(const TL<V>& level, V* xs, int gg, int NG, int lane, const XBars& xb, bool out) {
+  constexpr int NPF = tail_npf<D, V>();
+  constexpr bool LC = XM == X_CTA;
+  const TL<V> L = level;  // in registers: the asm statements' memory clobbers would have it loaded again at every step
   const int C = L.ncol;
-  auto colour = [&](int i) { return MODE == 0 ? i : C - 1 - i; };
-  RowPF<D, V, 1> cur;
-  {
-    const int c = colour(0), q0 = __ldg(L.cs + c), q1 = __ldg(L.cs + c + 1);
-    row_prefetch<D, G, V, S, MODE, TL<V>, LC>(L, q0 + gg, q0 + gg < q1, lane, cur);
+  const bool smem_cs = C <= TAIL_MAX_COLOURS;
+  if (smem_cs) {
+#pragma unroll 1
+    for (int i = threadIdx.x; i <= C; i += blockDim.x) xb.cs[i] = __ldg(L.cs + i);
+    __syncthreads();
   }
-  for (int i = 0; i < C; ++i) {
-    const int c = colour(i), r0 = __ldg(L.cs + c), r1 = __ldg(L.cs + c + 1);
-    for (int base = r0; base < r1; base += NG) {
-      RowPF<D, V, 1> nxt;
-      bool have = false;
-      if (base + NG < r1) {
-        row_prefetch<D, G, V, S, MODE, TL<V>, LC>(L, base + NG + gg, base + NG + gg < r1, lane, nxt);
-        have = true;
-      } else if (i + 1 < C) {
-        const int c2 = colour(i + 1), q0 = __ldg(L.cs + c2), q1 = __ldg(L.cs + c2 + 1);
-        row_prefetch<D, G, V, S, MODE, TL<V>, LC>(L, q0 + gg, q0 + gg < q1, lane, nxt);
-        have = true;
-      }
-      row_finish<D, G, V, S, MODE, TL<V>, LC>(L, base + gg, base + gg < r1, lane, cur);
-      if (have) cur = nxt;
+  // the rows [base, base + NG) of the i-th colour swept, and the ones after them
+  struct Pos {
+    int i, base, r1;
+  };
+  auto start = [&](int i) __attribute__((always_inline)) {
+    Pos q{i, 0, 0};
+    if (i < C) {
+      const int c = MODE == 0 ? i : C - 1 - i;
+      q.base = smem_cs ? xb.cs[c] : __ldg(L.cs + c);
+      q.r1 = smem_cs ? xb.cs[c + 1] : __ldg(L.cs + c + 1);
     }
-    sync();
+    return q;
+  };
+  auto after = [&](const Pos& p) __attribute__((always_inline)) {
+    if (p.base + NG < p.r1) return Pos{p.i, p.base + NG, p.r1};
+    return start(p.i + 1);
+  };
+  auto range = [&](const Pos& p) __attribute__((always_inline)) {
+    RowSeg r{0, 0, 0, 0};
+    if (p.base + gg < p.r1) r = seg_range<MODE>(L, p.base + gg);
+    return r;
+  };
+  if constexpr (XM == X_CLUSTER) {
+#pragma unroll 1
+    for (int i = threadIdx.x; i < xb.nbar; i += blockDim.x) {
+      const Pos q = start(i);
+      mbar_arrive_tx(xb.bar + i, (unsigned)((q.r1 - q.base) * xs_bytes<D, V>()));
+    }
   }
+  const int own = own_comp<D, G>(lane);
+  const bool leader = own < D && (lane & (own_step<D, G>() - 1)) == 0;
+  TailRow<D, V, S, NPF> sa{}, sb{};
+  auto load = [&](const Pos& p, const RowSeg& g, TailRow<D, V, S, NPF>& st) __attribute__((always_inline)) {
+    if (p.i < C) tail_row_load<D, G, V, S, MODE, LC>(L, p.base + gg, p.base + gg < p.r1, lane, g, st);
+  };
+  Pos cur = start(0), nxt = after(cur), nn = nxt.i < C ? after(nxt) : nxt;
+  load(cur, range(cur), sa);
+  load(nxt, range(nxt), sb);
+  RowSeg sg = range(nn);
+  // the row at `cur`, then the entries of the one two ahead into its registers
+  auto step = [&](TailRow<D, V, S, NPF>& st) __attribute__((always_inline)) {
+    const int row = cur.base + gg;
+    const bool valid = row < cur.r1;
+    if (__any_sync(0xffffffffu, valid)) {
+      const V v = tail_row_value<D, G, V, S, MODE, XM>(L, xs, lane, st);
+      if constexpr (XM == X_CLUSTER) {
+        V all[D];
+#pragma unroll
+        for (int a = 0; a < D; ++a) all[a] = __shfl_sync(0xffffffffu, v, a * own_step<D, G>(), G);
+        if (valid)
+#pragma unroll 1
+          for (int r = lane; r < xb.nct; r += G)
+            xs_send<D, V>(smem_u32(xs + row * xs_stride<D, V>()), smem_u32(xb.bar + cur.i), (unsigned)r, all);
+        if (out && valid && leader) stx<false>(L.x + (long long)row * D + own, v);
+      } else {
+        if (valid && leader) stx<LC>(L.x + (long long)row * D + own, v);
+      }
+    }
+    const bool last = nxt.i != cur.i;  // of its colour
+    if (XM == X_GLOBAL && last) asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
+    load(nn, sg, st);
+    const int done = cur.i;
+    cur = nxt;
+    nxt = nn;
+    if (nn.i < C) {
+      nn = after(nn);
+      sg = range(nn);
+    }
+    if (last) {
+      if (XM == X_GLOBAL) asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+      if (XM == X_CTA) __syncthreads();
+      if (XM == X_CLUSTER) mbar_wait(xb.bar + done, xb.parity, xb.abort);
+    }
+  };
+#pragma unroll 1
+  while (cur.i < C) {
+    step(sa);
+    if (cur.i >= C) break;
+    step(sb);
+  }
+}
+
+// r = -(upper part) x of a tail level, the next two rows' entries, and the range
+// of the one after them, in flight while the current row's x is gathered.
+template <int D, int G, typename V, typename S, int XM>
+__device__ __forceinline__ void tail_residual(const TL<V>& level, const V* xs, int gg, int NG, int lane) {
+  constexpr bool LC = XM == X_CTA;
+  const TL<V> L = level;
+  TailRow<D, V, S, 2> s0{}, s1{}, s2{};
+  const int own = own_comp<D, G>(lane);
+  const bool leader = own < D && (lane & (own_step<D, G>() - 1)) == 0;
+  RowSeg sg{0, 0, 0, 0};
+  auto range = [&](int row) __attribute__((always_inline)) {
+    sg = RowSeg{0, 0, 0, 0};
+    if (row < L.nv) sg = seg_range<2>(L, row);
+  };
+  // the entries of `row`, whose range is in sg, then the range of the group's next row
+  auto load = [&](int row, TailRow<D, V, S, 2>& st) __attribute__((always_inline)) {
+    tail_row_load<D, G, V, S, 2, LC>(L, row, row < L.nv, lane, sg, st);
+    range(row + NG);
+  };
+  auto finish = [&](int row, const TailRow<D, V, S, 2>& st) __attribute__((always_inline)) {
+    if (!__any_sync(0xffffffffu, row < L.nv)) return;
+    const V v = tail_row_value<D, G, V, S, 2, XM>(L, xs, lane, st);
+    if (row < L.nv && leader) stx<LC>(L.r + (long long)row * D + own, v);
+  };
+  range(gg);
+  load(gg, s0);
+  load(gg + NG, s1);
+#pragma unroll 1
+  for (int row = gg; __any_sync(0xffffffffu, row < L.nv); row += 3 * NG) {
+    load(row + 2 * NG, s2);
+    finish(row, s0);
+    load(row + 3 * NG, s0);
+    finish(row + NG, s1);
+    load(row + 4 * NG, s1);
+    finish(row + 2 * NG, s2);
+  }
+}
+
+// x_l += P x_{l+1} on a level whose x every CTA of the cluster holds: thread per
+// row, the new values to the level's copy in global memory (tail_fetch_xs then
+// brings them into every CTA; storing them straight into 16 CTAs' shared
+// memory took 4 times as long).  x_{l+1} from this CTA's copy (xsc) or global
+// memory; the sum in the order of prolong_row.
+template <int D, typename V>
+__device__ __forceinline__ void tail_prolong_xs(const TL<V>& L, const V* xs, const V* xsc, int tid, int NT) {
+  for (int i = tid; i < L.nv; i += NT) {
+    const int t0 = __ldg(L.prp + i), t1 = __ldg(L.prp + i + 1);
+    const uint8_t dm = __ldg(L.dead + i);
+    V acc[D];
+#pragma unroll
+    for (int a = 0; a < D; ++a) acc[a] = V(0);
+    constexpr int U = 1 << D;  // entries of a row of P at most
+    for (int t = t0; t < t1; t += U) {
+      V w[U], x[U][D];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        w[u] = V(0);
+#pragma unroll
+        for (int a = 0; a < D; ++a) x[u][a] = V(0);
+        if (t + u < t1) {
+          const int J = __ldg(L.pci + t + u);
+          w[u] = __ldg((const V*)L.pw + t + u);
+          if (xsc) xs_gather<D, V>(xsc, J, x[u]);
+          else ldx_vertex<D, false, true, false>((const V*)L.xc + (long long)J * D, x[u]);
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (t + u < t1) {
+#pragma unroll
+          for (int a = 0; a < D; ++a) acc[a] += w[u] * x[u][a];
+        }
+    }
+    V v[D];
+    xs_gather<D, V>(xs, i, v);
+#pragma unroll
+    for (int a = 0; a < D; ++a)
+      if (!((dm >> a) & 1)) v[a] += acc[a];
+    V* o = L.xg + (long long)i * xs_stride<D, V>();
+    if constexpr (sizeof(V) == 4) {
+      if constexpr (D == 2) __stcg(reinterpret_cast<float2*>(o), make_float2(v[0], v[1]));
+      else __stcg(reinterpret_cast<float4*>(o), make_float4(v[0], v[1], v[2], 0.0f));
+    } else {
+#pragma unroll
+      for (int a = 0; a < D; ++a) __stcg(o + a, v[a]);
+    }
+  }
+}
+template <int D, typename V>
+__device__ __forceinline__ void tail_fetch_xs(const TL<V>& L, V* xs) {
+  const float4* g = reinterpret_cast<const float4*>(L.xg);
+  float4* o = reinterpret_cast<float4*>(xs);
+  const int n16 = (L.nv * xs_bytes<D, V>() + 15) / 16;  // both copies are padded to 16 bytes
+#pragma unroll 4
+  for (int t = threadIdx.x; t < n16; t += blockDim.x) o[t] = __ldcg(g + t);
+  __syncthreads();
 }
 
 // Level l of the one-CTA part with its vectors in shared memory: x, b, r of
@@ -1279,11 +1679,13 @@ __device__ __forceinline__ void one_cta_down(const TailArgs<V>& A, V* sm, int lf
   constexpr int G = tail_g<D>();
   const int ng = blockDim.x / G, g = (int)threadIdx.x / G, lane = threadIdx.x & (G - 1);
   const int tid = threadIdx.x, NT = blockDim.x;
+  __shared__ int colour_start[TAIL_MAX_COLOURS + 1];
+  XBars xb{};
+  xb.cs = colour_start;
   for (int l = lfrom; l < lto; ++l) {
     const TL<V> L = shared_level<D, V>(A, l, sm);
-    tail_sweep<D, G, V, S, 0, true>(L, g, ng, lane, CtaSync());
-    for (int base = 0; base < L.nv; base += ng)
-      row_pass<D, G, V, S, 2, TL<V>, true>(L, base + g, base + g < L.nv, lane);
+    tail_sweep<D, G, V, S, 0, X_CTA>(L, L.x, g, ng, lane, xb, false);
+    tail_residual<D, G, V, S, X_CTA>(L, L.x, g, ng, lane);
     __syncthreads();
     for (int I = tid; I < L.nvc; I += NT) restrict_row<D, V, TL<V>, true>(L, I);
     __syncthreads();
@@ -1297,18 +1699,21 @@ __device__ __forceinline__ void one_cta_up(const TailArgs<V>& A, V* sm, int lfro
   constexpr int G = tail_g<D>();
   const int ng = blockDim.x / G, g = (int)threadIdx.x / G, lane = threadIdx.x & (G - 1);
   const int tid = threadIdx.x, NT = blockDim.x;
+  __shared__ int colour_start[TAIL_MAX_COLOURS + 1];
+  XBars xb{};
+  xb.cs = colour_start;
   for (int l = lfrom - 1; l >= lto; --l) {
     const TL<V> L = shared_level<D, V>(A, l, sm);
     for (int i = tid; i < L.nv; i += NT) prolong_row<D, V, TL<V>, true>(L, i);
     __syncthreads();
-    tail_sweep<D, G, V, S, 1, true>(L, g, ng, lane, CtaSync());
+    tail_sweep<D, G, V, S, 1, X_CTA>(L, L.x, g, ng, lane, xb, false);
   }
 }
 
 // Levels ls..L of the V-cycle on one CTA: phases separated by CTA barriers,
 // only b_ls comes in and x_ls goes out.
 template <int D, typename V, typename S>
-__device__ void tail_one_cta(const TailArgs<V>& A) {
+__device__ __forceinline__ void tail_one_cta(const TailArgs<V>& A) {
   extern __shared__ __align__(16) unsigned char tail_smem[];
   V* sm = reinterpret_cast<V*>(tail_smem);
   const int tid = threadIdx.x, NT = blockDim.x;
@@ -1347,7 +1752,7 @@ __device__ __forceinline__ void dense_level_rows(const TailArgs<float>& A, float
   for (int t = rank * wpc + ((int)threadIdx.x >> 5); t < n; t += nw) {
     const float4* m4 = reinterpret_cast<const float4*>(A.dm + (long long)t * ld);
     float a0 = 0.0f, a1 = 0.0f, a2 = 0.0f, a3 = 0.0f;
-#pragma unroll 4
+#pragma unroll 8
     for (int j = lane; j < ld4; j += 32) {
       const float4 mv = __ldg(m4 + j), bv = sb4[j];
       a0 += mv.x * bv.x;
@@ -1362,75 +1767,89 @@ __device__ __forceinline__ void dense_level_rows(const TailArgs<float>& A, float
   }
 }
 
-// The one-CTA part with a dense level kd: levels ls..kd-1 on CTA 0, then
-// x_kd = M b_kd on the whole cluster, then back up on CTA 0.  b_kd and x_kd
-// pass between the CTAs through global memory across cluster barriers.
-template <int D, typename V, typename S>
-__device__ void tail_dense_part(const TailArgs<V>& A, int rank, int nct) {
-  extern __shared__ __align__(16) unsigned char tail_smem[];
-  V* sm = reinterpret_cast<V*>(tail_smem);
-  const int ls = A.ls, kd = A.kd, n_ls = A.lv[ls].nv * D, n_kd = A.dn;
-  if (rank == 0 && kd > ls) {
-    const TL<V> Ls = shared_level<D, V>(A, ls, sm);
-    for (int t = threadIdx.x; t < n_ls; t += blockDim.x) Ls.b[t] = __ldcg(A.lv[ls].b + t);
-    __syncthreads();
-    one_cta_down<D, V, S>(A, sm, ls, kd);
-    const TL<V> Lk = shared_level<D, V>(A, kd, sm);
-    for (int t = threadIdx.x; t < n_kd; t += blockDim.x) __stcg(A.lv[kd].b + t, Lk.b[t]);
-  }
-  cluster_sync_all();
-  dense_level_rows(A, sm + A.dsoff, rank, nct);
-  cluster_sync_all();
-  if (rank == 0 && kd > ls) {
-    const TL<V> Lk = shared_level<D, V>(A, kd, sm);
-    for (int t = threadIdx.x; t < n_kd; t += blockDim.x) Lk.x[t] = __ldcg(A.lv[kd].x + t);
-    __syncthreads();
-    one_cta_up<D, V, S>(A, sm, kd, ls);
-    const TL<V> Ls = shared_level<D, V>(A, ls, sm);
-    for (int t = threadIdx.x; t < n_ls; t += blockDim.x) __stcg(A.lv[ls].x + t, Ls.x[t]);
-  }
-}
-
-// The V-cycle of all small levels in one cluster of CTAs, phases separated by
-// hardware cluster barriers; every group runs the same number of loop trips
-// so the sub-warp shuffles stay converged.  The smallest levels (ls..L) run
-// on CTA 0 alone between two cluster barriers.
+// The V-cycle of all small levels in one cluster of CTAs.  Levels l0..ls-1 run
+// on the whole cluster, the ones whose x fits with a copy of it in every CTA's
+// shared memory; rows are dealt to the CTAs first and then to their warps, so
+// that a colour of a few dozen rows spreads over all of them.  The levels below
+// are the dense level's product, or run on CTA 0 alone between two cluster
+// barriers.  Every group runs the same number of loop trips so the shuffles
+// stay converged.
 template <int D, typename V, typename S>
 __device__ __forceinline__ void tail_run(const TailArgs<V>& A) {
+  extern __shared__ __align__(16) unsigned char tail_smem[];
+  __shared__ __align__(8) unsigned long long xbar[TAIL_MAX_COLOURS];
+  __shared__ int colour_start[TAIL_MAX_COLOURS + 1];
+  // the current level's pointers
+  __shared__ __align__(16) unsigned char level_mem[sizeof(TL<V>)];
+  const TL<V>& L = *reinterpret_cast<const TL<V>*>(level_mem);
+  auto set_level = [&](int l) {
+    __syncthreads();
+    for (int i = threadIdx.x; i < (int)(sizeof(TL<V>) / 4); i += blockDim.x)
+      reinterpret_cast<unsigned*>(level_mem)[i] = reinterpret_cast<const unsigned*>(&A.lv[l])[i];
+    __syncthreads();
+  };
+  V* sm = reinterpret_cast<V*>(tail_smem);
   constexpr int G = tail_g<D>();
   const int nct = (int)cluster_size(), rank = (int)cluster_rank();
-  const int ng = blockDim.x / G;
-  const int gg = rank * ng + (int)threadIdx.x / G, NG = nct * ng;
+  const int NG = nct * ((int)blockDim.x / G);
+  const int gg = (((int)threadIdx.x >> 5) * nct + rank) * (32 / G) + ((int)threadIdx.x & 31) / G;
   const int lane = threadIdx.x & (G - 1);
   const int tid = rank * blockDim.x + threadIdx.x, NT = nct * blockDim.x;
+  const int g4 = (((int)threadIdx.x >> 5) * nct + rank) * 8 + ((int)threadIdx.x & 31) / 4;
   const int l0 = A.l0, ls = A.ls;
+  XBars xb{xbar, 0u, A.nbar, nct, A.abort, colour_start};
+  for (int i = threadIdx.x; i < A.nbar; i += blockDim.x) mbar_init(xbar + i, 1);
+  mbar_fence_init();
+  cluster_sync_all();
+#pragma unroll 1
   for (int l = l0; l < ls; ++l) {
-    const TL<V>& L = A.lv[l];
-    tail_sweep<D, G, V, S, 0, false>(L, gg, NG, lane, ClusterSync());
-    for (int base = 0; base < L.nv; base += NG) row_pass<D, G, V, S, 2>(L, base + gg, base + gg < L.nv, lane);
+    set_level(l);
+    if (L.xoff >= 0) {
+      tail_sweep<D, G, V, S, 0, X_CLUSTER>(L, sm + L.xoff, gg, NG, lane, xb, false);
+      xb.parity ^= 1u;
+      tail_residual<D, G, V, S, X_CLUSTER>(L, sm + L.xoff, gg, NG, lane);
+    } else {
+      tail_sweep<D, G, V, S, 0, X_GLOBAL>(L, nullptr, gg, NG, lane, xb, true);
+      tail_residual<D, G, V, S, X_GLOBAL>(L, nullptr, gg, NG, lane);
+    }
     cluster_sync_all();
-    for (int I = tid; I < L.nvc; I += NT) restrict_row<D, V>(L, I);
+    for (int base = 0; base < L.nvc; base += NT / 4) {
+      const int I = base + g4;
+      restrict_row_g4<D, V>(L, I, I < L.nvc, (int)threadIdx.x & 3);
+    }
     cluster_sync_all();
   }
   if constexpr (std::is_same<V, float>::value) {
     if (A.kd >= 0)
-      tail_dense_part<D, V, S>(A, rank, nct);
+      dense_level_rows(A, sm + A.dsoff, rank, nct);
     else if (rank == 0)
       tail_one_cta<D, V, S>(A);
   } else {
     if (rank == 0) tail_one_cta<D, V, S>(A);
   }
   cluster_sync_all();
+#pragma unroll 1
   for (int l = ls - 1; l >= l0; --l) {
-    const TL<V>& L = A.lv[l];
-    for (int i = tid; i < L.nv; i += NT) prolong_row<D, V>(L, i);
-    cluster_sync_all();
-    tail_sweep<D, G, V, S, 1, false>(L, gg, NG, lane, ClusterSync());
+    set_level(l);
+    const V* xsc = l + 1 < ls && A.lv[l + 1].xoff >= 0 ? sm + A.lv[l + 1].xoff : nullptr;
+    if (L.xoff >= 0) {
+      tail_prolong_xs<D, V>(L, sm + L.xoff, xsc, tid, NT);
+      cluster_sync_all();
+      tail_fetch_xs<D, V>(L, sm + L.xoff);
+      tail_sweep<D, G, V, S, 1, X_CLUSTER>(L, sm + L.xoff, gg, NG, lane, xb, l == l0 || A.lv[l - 1].xoff < 0);
+      xb.parity ^= 1u;
+    } else {
+      for (int i = tid; i < L.nv; i += NT) prolong_row<D, V>(L, i);
+      cluster_sync_all();
+      tail_sweep<D, G, V, S, 1, X_GLOBAL>(L, nullptr, gg, NG, lane, xb, true);
+    }
   }
+  // no CTA leaves while another may still send to it
+  cluster_sync_all();
 }
 
 template <int D, typename V, typename S>
-__global__ void __launch_bounds__(TAIL_THREADS) tail_kernel(const __grid_constant__ TailArgs<V> A) {
+__global__ void __launch_bounds__(tail_threads<D, V>(), 1) tail_kernel(const __grid_constant__ TailArgs<V> A) {
   tail_run<D, V, S>(A);
 }
 
@@ -1438,7 +1857,7 @@ __global__ void __launch_bounds__(TAIL_THREADS) tail_kernel(const __grid_constan
 // from level kd (= A.ls) on the unit vector e_j, with its own coarse-solve
 // scratch, and writes the result to column j of M (row-major, n x n).
 template <int D, typename V, typename S>
-__global__ void __launch_bounds__(TAIL_THREADS) dense_level_kernel(const __grid_constant__ TailArgs<V> A, V* M,
+__global__ void __launch_bounds__(tail_threads<D, V>(), 1) dense_level_kernel(const __grid_constant__ TailArgs<V> A, V* M,
                                                                    double* yscratch) {
   extern __shared__ __align__(16) unsigned char tail_smem[];
   V* sm = reinterpret_cast<V*>(tail_smem);
@@ -1726,7 +2145,8 @@ struct EngineView {
   std::vector<i64> nv;             // vertices per level
   std::vector<double> pnnz;        // transfer entries of level l -> l+1
   TailArgs<V> ta;                  // the tail launch from level lt (dense level fields set if used)
-  size_t tail_smem = 0;            // its dynamic shared memory, without the staging of b_kd
+  size_t tail_smem = 0;            // its dynamic shared memory
+  size_t tail_smem_base = 0;       // the part before the staging of b_kd
   CGArgs cga;                      // level-0 FP64 operator (SELL), permutation, Dirichlet data
   int cg_blocks = 1, spmv_blocks = 1;
   i64 sell_real_entries = 0;

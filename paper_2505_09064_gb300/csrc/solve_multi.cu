@@ -593,56 +593,18 @@ __device__ __forceinline__ void dense_rows_m(const TailArgs<float>& A, float* sb
   }
 }
 
-// The one-CTA part with a dense level kd (FP32): levels ls..kd-1 on CTA 0 for
-// each right-hand side in turn (their shared vectors saved to `stash` for the
-// way up), x_kd = M b_kd for all of them on the cluster, then back up on CTA
-// 0 one right-hand side at a time.
-template <int D, int KR, typename S>
-__device__ void tailm_dense_part(const TailArgs<float>& A, int rank, int nct, float* stash) {
-  extern __shared__ __align__(16) unsigned char tail_smem[];
-  float* sm = reinterpret_cast<float*>(tail_smem);
-  const int ls = A.ls, kd = A.kd, n_ls = A.lv[ls].nv * D, n_kd = A.dn;
-  const int s0 = A.soff[ls], s1 = A.soff[kd], slen = s1 - s0;
-  if (rank == 0 && kd > ls) {
-    for (int i = 0; i < KR; ++i) {
-      const TL<float> Ls = shared_level<D, float>(A, ls, sm);
-      for (int t = threadIdx.x; t < n_ls; t += blockDim.x) Ls.b[t] = __ldcg(A.lv[ls].b + mix<D, KR>(t, i));
-      __syncthreads();
-      one_cta_down<D, float, S>(A, sm, ls, kd);
-      const TL<float> Lk = shared_level<D, float>(A, kd, sm);
-      for (int t = threadIdx.x; t < n_kd; t += blockDim.x) __stcg(A.lv[kd].b + mix<D, KR>(t, i), Lk.b[t]);
-      for (int t = threadIdx.x; t < slen; t += blockDim.x) stash[(long long)i * slen + t] = sm[s0 + t];
-      __syncthreads();
-    }
-  }
-  cluster_sync_all();
-  dense_rows_m<D, KR>(A, sm + A.dsoff, rank, nct);
-  cluster_sync_all();
-  if (rank == 0 && kd > ls) {
-    for (int i = 0; i < KR; ++i) {
-      for (int t = threadIdx.x; t < slen; t += blockDim.x) sm[s0 + t] = stash[(long long)i * slen + t];
-      const TL<float> Lk = shared_level<D, float>(A, kd, sm);
-      for (int t = threadIdx.x; t < n_kd; t += blockDim.x) Lk.x[t] = __ldcg(A.lv[kd].x + mix<D, KR>(t, i));
-      __syncthreads();
-      one_cta_up<D, float, S>(A, sm, kd, ls);
-      const TL<float> Ls = shared_level<D, float>(A, ls, sm);
-      for (int t = threadIdx.x; t < n_ls; t += blockDim.x) __stcg(A.lv[ls].x + mix<D, KR>(t, i), Ls.x[t]);
-      __syncthreads();
-    }
-  }
-}
-
 // The V-cycle of the small levels for KR right-hand sides: the cluster levels
 // with all of them at once, the one-CTA levels one right-hand side at a time,
 // the dense level for all at once.
 template <int D, int KR, typename S>
-__global__ void __launch_bounds__(TAILM_THREADS) tailm_kernel(const __grid_constant__ TailArgs<float> A,
-                                                             float* stash) {
+__global__ void __launch_bounds__(TAILM_THREADS) tailm_kernel(const __grid_constant__ TailArgs<float> A) {
+  extern __shared__ __align__(16) unsigned char tail_smem[];
   using V = float;
   constexpr int G = tail_g<D>();
   const int nct = (int)cluster_size(), rank = (int)cluster_rank();
-  const int ng = blockDim.x / G;
-  const int gg = rank * ng + (int)threadIdx.x / G, NG = nct * ng;
+  // rows dealt to the CTAs first, then to their warps (as tail_run)
+  const int NG = nct * ((int)blockDim.x / G);
+  const int gg = (((int)threadIdx.x >> 5) * nct + rank) * (32 / G) + ((int)threadIdx.x & 31) / G;
   const int lane = threadIdx.x & (G - 1);
   const int tid = rank * blockDim.x + threadIdx.x, NT = nct * blockDim.x;
   const int l0 = A.l0, ls = A.ls;
@@ -659,7 +621,7 @@ __global__ void __launch_bounds__(TAILM_THREADS) tailm_kernel(const __grid_const
     cluster_sync_all();
   }
   if (A.kd >= 0) {
-    tailm_dense_part<D, KR, S>(A, rank, nct, stash);
+    dense_rows_m<D, KR>(A, reinterpret_cast<float*>(tail_smem) + A.dsoff, rank, nct);
   } else if (rank == 0) {
     for (int i = 0; i < KR; ++i) tailm_one_cta<D, KR, V, S>(A, i);
   }
@@ -919,7 +881,6 @@ struct MultiEngine : MultiBase {
   DevBuf<double> U, r, p, q, Fb, Ub, part, hist;
   DevBuf<Scalars> sc;
   DevBuf<int> ctl;
-  DevBuf<V> stash;
   Scalars* host_sc = nullptr;
   int* host_ctl = nullptr;
   int pstride = 1;
@@ -981,11 +942,6 @@ struct MultiEngine : MultiBase {
     sc.zero();
     ctl.alloc(2, s);
     ctl.zero();
-    // the one-CTA levels above the dense level, saved per right-hand side
-    const TailArgs<V>& ta = v.ta;
-    i64 slen = 1;
-    if (ta.kd > ta.ls) slen = ta.soff[ta.kd] - ta.soff[ta.ls];
-    stash.alloc(std::max<i64>(1, slen) * kr, s);
     if (!host_sc) VASMG_CUDA(cudaMallocHost((void**)&host_sc, sizeof(Scalars) * KMAX));
     if (!host_ctl) VASMG_CUDA(cudaMallocHost((void**)&host_ctl, sizeof(int) * 2));
     cap = kr;
@@ -1124,8 +1080,8 @@ struct MultiEngine : MultiBase {
   }
   template <int KR>
   size_t tail_smem_bytes() const {
-    size_t smem = v.tail_smem;
-    if (v.ta.kd >= 0 && v.ta.kd >= v.ta.ls) smem = (size_t)v.ta.dsoff * sizeof(V) + sizeof(V) * (size_t)KR * v.ta.dld;
+    size_t smem = v.tail_smem_base;
+    if (v.ta.kd >= 0) smem = (size_t)v.ta.dsoff * sizeof(V) + sizeof(V) * (size_t)KR * v.ta.dld;
     return smem;
   }
   template <int KR>
@@ -1155,7 +1111,7 @@ struct MultiEngine : MultiBase {
     at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    VASMG_CUDA(cudaLaunchKernelEx(&cfg, tailm_kernel<D, KR, S>, ta, stash.get()));
+    VASMG_CUDA(cudaLaunchKernelEx(&cfg, tailm_kernel<D, KR, S>, ta));
     ++launch_counter;
   }
   template <int KR>
@@ -1564,7 +1520,7 @@ __global__ void __launch_bounds__(DFM_THREADS) transferb_kernel(const BatchItem*
 // Every hierarchy's tail: cluster c runs hierarchy c's levels from its own
 // first tail level down and back.
 template <typename S>
-__global__ void __launch_bounds__(TAIL_THREADS) tailb_kernel(const TailArgs<float>* __restrict__ args,
+__global__ void __launch_bounds__(TAILB_THREADS, 1) tailb_kernel(const TailArgs<float>* __restrict__ args,
                                                              const int* __restrict__ dims) {
   const int c = blockIdx.x / (int)cluster_size();
   if (dims[c] == 2) tail_run<2, float, S>(args[c]);
@@ -1815,9 +1771,7 @@ struct BatchRun {
       maxlt = std::max(maxlt, e.lt);
       nct = std::max(nct, e.nct);
       max_iters = std::max(max_iters, e.max_iters);
-      size_t sm = e.tail_smem;
-      if (e.ta.kd >= 0 && e.ta.kd >= e.ta.ls) sm = (size_t)e.ta.dsoff * sizeof(float) + sizeof(float) * (size_t)e.ta.dld;
-      tail_smem = std::max(tail_smem, sm);
+      tail_smem = std::max(tail_smem, e.tail_smem);
     }
     const int cap = batch_sweep_capacity<S>();
     sweep_items.resize(maxlt);
@@ -1871,11 +1825,14 @@ struct BatchRun {
       restrict_ctas[l] = r0;
       prolong_ctas[l] = q0;
     }
+    abort_flag.alloc(1, s);
+    abort_flag.zero();
     std::vector<TailArgs<float>> ta(n);
     std::vector<int> dims(n);
     std::vector<CGB> cgh(n);
     for (int i = 0; i < n; ++i) {
       ta[i] = v[i].ta;
+      ta[i].abort = abort_flag.get();
       dims[i] = v[i].dim;
       CGB& m = cgh[i];
       m.a = v[i].cga;
@@ -1898,8 +1855,6 @@ struct BatchRun {
     cg.upload(cgh.data(), n);
     ctl.alloc(2, s);
     ctl.zero();
-    abort_flag.alloc(1, s);
-    abort_flag.zero();
     VASMG_CHECK(tail_smem <= (size_t)TAIL_SMEM_MAX, VASMG_ERR_UNSUPPORTED, "tail levels too large for shared memory");
     VASMG_CUDA(cudaFuncSetAttribute(tailb_kernel<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, TAIL_SMEM_MAX));
     if (nct > 8 && cudaFuncSetAttribute(tailb_kernel<S>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
@@ -1911,7 +1866,7 @@ struct BatchRun {
     while (nct > 1) {
       cudaLaunchConfig_t cfg = {};
       cfg.gridDim = dim3(nct);
-      cfg.blockDim = dim3(TAIL_THREADS);
+      cfg.blockDim = dim3(TAILB_THREADS);
       cfg.dynamicSmemBytes = tail_smem;
       cudaLaunchAttribute at[1];
       at[0].id = cudaLaunchAttributeClusterDimension;
@@ -1955,7 +1910,7 @@ struct BatchRun {
     {
       cudaLaunchConfig_t cfg = {};
       cfg.gridDim = dim3(nct * n);
-      cfg.blockDim = dim3(TAIL_THREADS);
+      cfg.blockDim = dim3(TAILB_THREADS);
       cfg.dynamicSmemBytes = tail_smem;
       cfg.stream = s;
       cudaLaunchAttribute at[1];
