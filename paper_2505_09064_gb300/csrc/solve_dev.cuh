@@ -1205,6 +1205,14 @@ __device__ __forceinline__ void seg_ptrs(const TL<V>& L, const int*& ciA, const 
   offA = offB = (const S*)L.off;
   nA = nB = L.nnz;
 }
+// The same as its two ends (a difference taken at once would wait for the loads)
+struct RowEnds {
+  int a0, a1;
+};
+template <int MODE, typename V>
+__device__ __forceinline__ RowEnds row_ends(const TL<V>& L, int row) {
+  return RowEnds{MODE == 2 ? __ldg(L.sp + row) : __ldg(L.rp + row), MODE == 0 ? __ldg(L.sp + row) : __ldg(L.rp + row + 1)};
+}
 template <int MODE, typename V>
 __device__ __forceinline__ RowSeg seg_range(const TL<V>& L, int row) {
   RowSeg r;
@@ -1380,15 +1388,15 @@ struct TailRow {
 };
 
 template <int D, int G, typename V, typename S, int MODE, bool LC, int NPF>
-__device__ __forceinline__ void tail_row_load(const TL<V>& L, int row, bool valid, int lane, const RowSeg& sg,
+__device__ __forceinline__ void tail_row_load(const TL<V>& L, int row, bool valid, int lane, const RowEnds& sg,
                                               TailRow<D, V, S, NPF>& st) {
   st.a0 = sg.a0;
-  st.len = sg.len;
+  st.len = sg.a1 - sg.a0;
 #pragma unroll
   for (int p = 0; p < NPF; ++p) {
     const int e = lane + p * G;
     st.col[p] = -1;
-    if (e < sg.len) {
+    if (e < st.len) {
       st.col[p] = __ldg(L.ci + sg.a0 + e);
       st.blk[p].load((const S*)L.off, L.nnz, sg.a0 + e);
     }
@@ -1494,8 +1502,8 @@ __device__ __forceinline__ void tail_sweep(const TL<V>& level, V* xs, int gg, in
     return start(p.i + 1);
   };
   auto range = [&](const Pos& p) __attribute__((always_inline)) {
-    RowSeg r{0, 0, 0, 0};
-    if (p.base + gg < p.r1) r = seg_range<MODE>(L, p.base + gg);
+    RowEnds r{0, 0};
+    if (p.base + gg < p.r1) r = row_ends<MODE>(L, p.base + gg);
     return r;
   };
   if constexpr (XM == X_CLUSTER) {
@@ -1508,13 +1516,13 @@ __device__ __forceinline__ void tail_sweep(const TL<V>& level, V* xs, int gg, in
   const int own = own_comp<D, G>(lane);
   const bool leader = own < D && (lane & (own_step<D, G>() - 1)) == 0;
   TailRow<D, V, S, NPF> sa{}, sb{};
-  auto load = [&](const Pos& p, const RowSeg& g, TailRow<D, V, S, NPF>& st) __attribute__((always_inline)) {
+  auto load = [&](const Pos& p, const RowEnds& g, TailRow<D, V, S, NPF>& st) __attribute__((always_inline)) {
     if (p.i < C) tail_row_load<D, G, V, S, MODE, LC>(L, p.base + gg, p.base + gg < p.r1, lane, g, st);
   };
   Pos cur = start(0), nxt = after(cur), nn = nxt.i < C ? after(nxt) : nxt;
   load(cur, range(cur), sa);
   load(nxt, range(nxt), sb);
-  RowSeg sg = range(nn);
+  RowEnds sg = range(nn);
   // the row at `cur`, then the entries of the one two ahead into its registers
   auto step = [&](TailRow<D, V, S, NPF>& st) __attribute__((always_inline)) {
     const int row = cur.base + gg;
@@ -1567,10 +1575,10 @@ __device__ __forceinline__ void tail_residual(const TL<V>& level, const V* xs, i
   TailRow<D, V, S, 2> s0{}, s1{}, s2{};
   const int own = own_comp<D, G>(lane);
   const bool leader = own < D && (lane & (own_step<D, G>() - 1)) == 0;
-  RowSeg sg{0, 0, 0, 0};
+  RowEnds sg{0, 0};
   auto range = [&](int row) __attribute__((always_inline)) {
-    sg = RowSeg{0, 0, 0, 0};
-    if (row < L.nv) sg = seg_range<2>(L, row);
+    sg = RowEnds{0, 0};
+    if (row < L.nv) sg = row_ends<2>(L, row);
   };
   // the entries of `row`, whose range is in sg, then the range of the group's next row
   auto load = [&](int row, TailRow<D, V, S, 2>& st) __attribute__((always_inline)) {
