@@ -308,6 +308,7 @@ struct Engine : EngineBase {
   std::vector<int> G;
   std::vector<DevBuf<int32_t>> cs_dev, rs_dev, nb_rp, nb;
   std::vector<DevBuf<unsigned long long>> pg_d, pg_u;
+  std::vector<DevBuf<uint4>> xt;  // 3D region levels: the staged sweeps' tagged values
   std::vector<i64> nnz_lo;        // lower-part (earlier colour) blocks per level
   std::vector<DevBuf<int32_t>> rpl_dev, rph_dev, cil_dev, cih_dev;
   std::vector<DevBuf<S>> offl_dev, offh_dev;
@@ -343,6 +344,8 @@ struct Engine : EngineBase {
     long long nslots = 0;
     DevBuf<int32_t> ci, goff, srow, step_nact;
     DevBuf<long long> step_off;
+    DevBuf<int2> hdr;
+    DevBuf<int4> rec;
     DevBuf<S> v8, v9;
     StagedOp<S> op{};
   };
@@ -470,6 +473,11 @@ struct Engine : EngineBase {
     v.nb = nb[l].get();
     v.pg_d = pg_d[l].get();
     v.pg_u = pg_u[l].get();
+    if constexpr (D == 3) {
+      xt[l].alloc(std::max<i64>(1, c->S[l].nv) * xt_words<V>(), s);
+      xt[l].zero();  // no launch's tag is 0
+      v.xt = xt[l].get();
+    }
   }
 
   // New operator values on the same structure: the level-0 FP64 SELL copy
@@ -547,6 +555,7 @@ struct Engine : EngineBase {
     rs_dev.resize(L);
     nb_rp.resize(L);
     nb.resize(L);
+    xt.resize(L);
     pg_d.resize(L);
     pg_u.resize(L);
     nnz_lo.assign(L, 0);
@@ -753,7 +762,9 @@ struct Engine : EngineBase {
         std::vector<long long> step_off((size_t)C * R + 1, 0);
         std::vector<int> step_nact((size_t)C * R, 32);
         std::vector<int> goff((size_t)C * R * (NG + 1), 0), srow(std::max(nv, 1), 0);
-        std::vector<int> order, load(NG), grp;
+        std::vector<int2> hdr((size_t)C * R);
+        std::vector<int4> rec((size_t)C * R * NG);
+        std::vector<int> order, load(NG);
         std::vector<std::vector<int>> lists(NG);
         for (int col = 0; col < C; ++col)
           for (int k = 0; k < R; ++k) {
@@ -775,14 +786,18 @@ struct Engine : EngineBase {
             int pos = r0, mx = 0, used = 0;
             for (int gi = 0; gi < NG; ++gi) {
               goff[step * (NG + 1) + gi] = pos - r0;
-              for (int r : lists[gi]) srow[pos++] = r;
+              const auto& rows = lists[gi];
+              const int nr = (int)rows.size();
+              rec[step * NG + gi] = make_int4(nr > 0 ? rows[0] : -1, nr > 1 ? rows[1] : -1, pos + 2, pos + nr);
+              for (int r : rows) srow[pos++] = r;
               mx = std::max(mx, load[gi]);
               if (!lists[gi].empty()) used = gi + 1;
             }
             goff[step * (NG + 1) + NG] = pos - r0;
             const int nact = std::min(STG_T, std::max(32, (int)ceil_div(used * g, 32) * 32));
             step_nact[step] = nact;
-            step_off[step + 1] = step_off[step] + ceil_div(mx, EPT) * EPT * nact;
+            hdr[step] = make_int2(nact, (int)ceil_div(mx, EPT));
+            step_off[step + 1] = step_off[step] + (i64)hdr[step].y * EPT * nact;
           }
         const i64 nslot = step_off[(size_t)C * R];
         st.step_off.alloc((i64)step_off.size(), s);
@@ -791,6 +806,10 @@ struct Engine : EngineBase {
         st.step_nact.upload(step_nact.data(), (i64)step_nact.size());
         st.goff.alloc((i64)goff.size(), s);
         st.goff.upload(goff.data(), (i64)goff.size());
+        st.hdr.alloc((i64)hdr.size(), s);
+        st.hdr.upload(hdr.data(), (i64)hdr.size());
+        st.rec.alloc((i64)rec.size(), s);
+        st.rec.upload(rec.data(), (i64)rec.size());
         st.srow.alloc((i64)srow.size(), s);
         st.srow.upload(srow.data(), (i64)srow.size());
         const i64 ne = std::max<i64>(STG_T * EPT, nslot);
@@ -805,7 +824,8 @@ struct Engine : EngineBase {
         st.op.v9 = st.v9.get();
         st.op.step_off = st.step_off.get();
         st.op.step_nact = st.step_nact.get();
-        st.op.goff = st.goff.get();
+        st.op.hdr = st.hdr.get();
+        st.op.rec = st.rec.get();
         st.op.srow = st.srow.get();
         st.G = g;
         fill_staged(l, m);
@@ -824,12 +844,13 @@ struct Engine : EngineBase {
     if (m == 0)
       stage_fill_kernel<S><<<grid_for(threads, 256), 256, 0, c->stream>>>(
           rpl_dev[l].get(), cil_dev[l].get(), offl_dev[l].get(), nnz_lo[l], lv[l].RS, lv[l].R, sl.ncol,
-          st.step_off.get(), st.step_nact.get(), st.goff.get(), st.srow.get(), st.G, st.ci.get(), st.v8.get(),
-          st.v9.get());
+          st.step_off.get(), st.step_nact.get(), st.goff.get(), st.srow.get(), st.G, m, st.ci.get(),
+          st.v8.get(), st.v9.get());
     else
       stage_fill_kernel<S><<<grid_for(threads, 256), 256, 0, c->stream>>>(
           sl.rp.get(), sl.ci.get(), (const S*)off_ptr(sl), sl.nnz, lv[l].RS, lv[l].R, sl.ncol, st.step_off.get(),
-          st.step_nact.get(), st.goff.get(), st.srow.get(), st.G, st.ci.get(), st.v8.get(), st.v9.get());
+          st.step_nact.get(), st.goff.get(), st.srow.get(), st.G, m, st.ci.get(), st.v8.get(),
+          st.v9.get());
     check_launch("stage_fill");
   }
   bool staged_on(int l) const {
@@ -918,6 +939,7 @@ struct Engine : EngineBase {
       VASMG_CUDA(cudaEventCreate(&e1));
       int best_g = G[l];
       float best_ms = 0.0f;
+      bool best_wide = true;
       for (int g : {4, 8, 16, 32}) {
         if (sweep_capacity(g) < lv[l].R) continue;
         G[l] = g;
@@ -934,9 +956,13 @@ struct Engine : EngineBase {
         VASMG_CUDA(cudaEventSynchronize(e1));
         float ms = 0.0f;
         VASMG_CUDA(cudaEventElapsedTime(&ms, e0, e1));
-        if (best_ms == 0.0f || ms < best_ms) {
+        // a staged copy of more than twice the level's blocks only where every
+        // choice needs one
+        const bool wide = stg[1].size() > (size_t)l && stg[1][l].G == g && stg[1][l].nslots > 2 * (i64)sl.nnz;
+        if (best_ms == 0.0f || (wide == best_wide ? ms < best_ms : best_wide)) {
           best_ms = ms;
           best_g = g;
+          best_wide = wide;
         }
       }
       cudaEventDestroy(e0);

@@ -238,6 +238,9 @@ struct LV {
   unsigned long long* pg_d;  // progress of each region in the down launch: epoch << 32 | stage
   unsigned long long* pg_u;  // same for the up launch
   int* ctr;               // C_N counters
+  // staged sweeps (3D): the values of the running launch with its tag, KR
+  // words per right-hand side and vertex (load_tagged)
+  uint4* xt;
 };
 
 template <int D>
@@ -793,9 +796,11 @@ __global__ void __launch_bounds__(256) prolong_kernel(const __grid_constant__ LV
 // the multi and batched sweeps).
 
 constexpr int STG_T = 256;  // consumer threads of a staged sweep CTA; one producer warp follows them
-// a slot: column in bits 0..29 (STG_NONE: no entry), STG_END: the row ends
-// with this slot; -1: padding after the thread's stream
-constexpr int STG_NONE = 0x3fffffff;
+// a slot: column in bits 0..28 (STG_NONE: no entry), STG_NEW: the sweep writes
+// the column before this row, STG_END: the row ends with this slot; -1:
+// padding after the thread's stream
+constexpr int STG_NONE = 0x1fffffff;
+constexpr int STG_NEW = 0x20000000;
 constexpr int STG_END = 0x40000000;
 
 // slots per consumer thread and chunk (as many gathers in flight): 4 with
@@ -821,8 +826,10 @@ struct StagedOp {
   const S* v9;                  // [EPT][nact] block component 8
   const long long* step_off;    // [ncol R + 1]: first slot of colour c in region k (step c R + k)
   const int* step_nact;         // [ncol R]: consumer threads the step's chunks hold (a multiple of 32)
-  const int* goff;              // [ncol R][NG + 1]: rows of group g in a step: srow[r0 + goff[g] .. r0 + goff[g + 1])
-  const int* srow;              // [nv]: each step's rows [r0, r1), group by group
+  const int2* hdr;              // [ncol R]: (consumer threads of a chunk, chunks) of a step
+  const int4* rec;              // [ncol R][NG]: group g's rows of a step: the first two (-1: none), then the third
+                                // and those after it, srow[z .. w)
+  const int* srow;              // [nv]: each step's rows, group by group
 };
 
 __device__ __forceinline__ unsigned smem_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
@@ -967,6 +974,141 @@ __device__ __forceinline__ void stg_row_data(const LV<V>& L, int row, bool load,
   }
 }
 
+// What a consumer knows of the colour step it is about to take.  A step's
+// rows and their data are a chain of loads, and the acquire of every neighbour
+// wait leaves none of it in L1.  So one record holds a group's first rows, and
+// that of step i + 1 is in flight while step i runs: D^-1 and b of step i are
+// then asked for before its neighbour wait.
+struct StgStep {
+  int2 h;  // threads of a chunk, chunks
+  int4 g;  // StagedOp::rec
+};
+template <int MODE, typename S>
+__device__ __forceinline__ StgStep stg_step(const StagedOp<S>& O, int i, int k, int R, int C, int NG, int g) {
+  StgStep st{make_int2(32, 0), make_int4(-1, -1, 0, 0)};
+  if (i < C) {
+    const int step = (MODE == 0 ? i : C - 1 - i) * R + k;
+    st.h = __ldg(O.hdr + step);
+    st.g = __ldg(O.rec + (long long)step * NG + g);
+  }
+  return st;
+}
+
+// ---- values with tags
+//
+// A staged sweep writes each vertex twice: into x, and into xt as 16-byte
+// words of 12 bytes of values and a 4-byte tag that names the launch.  A row
+// that needs a neighbour's new value reads that word until it carries the
+// launch's tag.  Value and tag are one 16-byte access (.b128, single-copy
+// atomic), so nothing orders them: no fence, no stage to publish, no barrier
+// between the colours, and a row waits for its own neighbours only.
+//
+// What the regions' stage waits cost before (clock stamps per colour step,
+// 33^3 FP32 level 1, forward): 7400 of 11,300 cycles in the neighbour wait,
+// 1900 in the release, 1600 on the rows themselves.
+//
+// Old values (backward sweep, columns the sweep writes after this row) come
+// from x through L1.  They are safe without a wait: the pattern is symmetric,
+// so the row that overwrites such a column waits for this row's new value,
+// which depends on everything this row has read.
+//
+// Every wait ends: rows wait only for rows of earlier colours, the producer
+// only for chunks before it, and each wait is bounded.
+template <typename V>
+constexpr int xt_words() { return (int)sizeof(V) / 4; }  // 16-byte words per vertex of 3 values
+
+__device__ __forceinline__ void ld_word(const uint4* p, unsigned (&u)[4]) {
+  asm volatile(
+      "{\n\t.reg .b128 t;\n\t.reg .b64 lo, hi;\n\tld.relaxed.gpu.global.b128 t, [%4];\n\tmov.b128 {lo, hi}, t;\n\t"
+      "mov.b64 {%0, %1}, lo;\n\tmov.b64 {%2, %3}, hi;\n\t}"
+      : "=r"(u[0]), "=r"(u[1]), "=r"(u[2]), "=r"(u[3])
+      : "l"(p));
+}
+__device__ __forceinline__ void st_word(uint4* p, unsigned a, unsigned b, unsigned c, unsigned tag) {
+  asm volatile(
+      "{\n\t.reg .b128 t;\n\t.reg .b64 lo, hi;\n\tmov.b64 lo, {%1, %2};\n\tmov.b64 hi, {%3, %4};\n\t"
+      "mov.b128 t, {lo, hi};\n\tst.relaxed.gpu.global.b128 [%0], t;\n\t}" ::"l"(p),
+      "r"(a), "r"(b), "r"(c), "r"(tag)
+      : "memory");
+}
+// 3 values as words: FP32 (v0, v1, v2, tag); FP64 (v0, low half of v1, tag)
+// and (v2, high half of v1, tag)
+__device__ __forceinline__ void st_tagged(uint4* p, float v0, float v1, float v2, unsigned tag) {
+  st_word(p, __float_as_uint(v0), __float_as_uint(v1), __float_as_uint(v2), tag);
+}
+__device__ __forceinline__ void st_tagged(uint4* p, double v0, double v1, double v2, unsigned tag) {
+  st_word(p, (unsigned)__double2loint(v0), (unsigned)__double2hiint(v0), (unsigned)__double2loint(v1), tag);
+  st_word(p + 1, (unsigned)__double2loint(v2), (unsigned)__double2hiint(v2), (unsigned)__double2hiint(v1), tag);
+}
+__device__ __forceinline__ void tagged_values(const unsigned (&u)[1][4], float (&x)[3]) {
+#pragma unroll
+  for (int a = 0; a < 3; ++a) x[a] = __uint_as_float(u[0][a]);
+}
+__device__ __forceinline__ void tagged_values(const unsigned (&u)[2][4], double (&x)[3]) {
+  x[0] = __hiloint2double((int)u[0][1], (int)u[0][0]);
+  x[1] = __hiloint2double((int)u[1][2], (int)u[0][2]);
+  x[2] = __hiloint2double((int)u[1][1], (int)u[1][0]);
+}
+// the values of x as words
+__device__ __forceinline__ void plain_words(const float* x, unsigned tag, unsigned (&u)[1][4]) {
+#pragma unroll
+  for (int a = 0; a < 3; ++a) u[0][a] = __float_as_uint(__ldca(x + a));
+  u[0][3] = tag;
+}
+__device__ __forceinline__ void plain_words(const double* x, unsigned tag, unsigned (&u)[2][4]) {
+  const double v0 = __ldca(x), v1 = __ldca(x + 1), v2 = __ldca(x + 2);
+  u[0][0] = (unsigned)__double2loint(v0), u[0][1] = (unsigned)__double2hiint(v0);
+  u[0][2] = (unsigned)__double2loint(v1), u[1][2] = (unsigned)__double2hiint(v1);
+  u[1][0] = (unsigned)__double2loint(v2), u[1][1] = (unsigned)__double2hiint(v2);
+  u[0][3] = u[1][3] = tag;
+}
+// Reads word p again until it carries the tag.  Gives up as mbar_wait does,
+// and at once when an earlier wait of this thread did (dead).
+__device__ __forceinline__ void wait_word(const uint4* p, unsigned tag, unsigned (&u)[4], int* abort_flag, bool& dead) {
+#pragma unroll 1
+  for (int spins = 0; u[3] != tag && !dead; ++spins) {
+    if (spins >= SPIN_LIMIT) {
+      atomicExch(abort_flag, 1);
+      dead = true;
+    }
+    if ((spins & 255) == 255 && *(volatile int*)abort_flag) dead = true;
+    if (spins >= 8) __nanosleep(32);
+    ld_word(p, u);
+  }
+}
+// Reads the words of NS slots again (word w of slot h at base + col(v[h]) W + w,
+// the slots of mask `tagged`) until all carry the tag: what is still missing is
+// asked for at once, so a row waits one round trip after its last neighbour
+// and not one per neighbour.  Gives up as wait_word does.
+template <int NS, int W>
+__device__ __forceinline__ void wait_words(const uint4* base, const int (&v)[NS], unsigned tagged, unsigned tag,
+                                           unsigned (&u)[NS][W][4], int* abort_flag, bool& dead) {
+#pragma unroll 1
+  for (int spins = 0; !dead; ++spins) {
+    bool miss = false;
+#pragma unroll
+    for (int h = 0; h < NS; ++h)
+#pragma unroll
+      for (int w = 0; w < W; ++w) miss |= (tagged >> h & 1u) && u[h][w][3] != tag;
+    if (!miss) return;
+    if (spins >= SPIN_LIMIT) {
+      atomicExch(abort_flag, 1);
+      dead = true;
+    }
+    if ((spins & 255) == 255 && *(volatile int*)abort_flag) dead = true;
+    if (spins >= 8) __nanosleep(32);
+#pragma unroll
+    for (int h = 0; h < NS; ++h)
+#pragma unroll
+      for (int w = 0; w < W; ++w)
+        if ((tagged >> h & 1u) && u[h][w][3] != tag)
+          ld_word(base + (long long)(v[h] & STG_NONE) * W + w, u[h][w]);
+  }
+}
+// The tag of this launch: the epoch counters of the two directions start at 1.
+template <int MODE>
+__device__ __forceinline__ unsigned sweep_tag(unsigned epoch) { return 2u * epoch + (unsigned)MODE; }
+
 // The consumers: region k's rows colour by colour, each group of G lanes
 // through its rows' slots, chunk by chunk from the ring.
 template <int D, int G, typename V, typename S, int MODE>
@@ -978,56 +1120,73 @@ __device__ __forceinline__ void stg_consume(const LV<V>& L, const StagedOp<S>& O
   const int tid = threadIdx.x, g = tid / G, lane = tid & (G - 1);
   // the lanes of this group within the warp
   const unsigned gmask = G == 32 ? 0xffffffffu : (((1u << G) - 1u) << ((tid & 31) & ~(G - 1)));
-  const int nb0 = __ldg(L.nb_rp + k), nnb = __ldg(L.nb_rp + k + 1) - nb0;
-  unsigned long long* pg = MODE == 0 ? L.pg_d : L.pg_u;
-  long long q = 0;  // chunks taken
+  constexpr int W = xt_words<V>();
+  // The waits of a chunk: slot after slot, each before its product, or for
+  // all its slots first.  Polling slot after slot loads L2 less (64^3 FP32
+  // level 1, 32 lanes: forward 169 against 234 us, backward 210 against 219);
+  // with at most 8 lanes the backward sweep's rows are many and mostly ready,
+  // and what is missing is better fetched together (128^3 BF16 level 1, 8
+  // lanes: 753 against 720 us; forward 522 against 554).
+  constexpr bool AT_ONCE = MODE == 1 && G <= 8;
+  const unsigned tag = sweep_tag<MODE>(epoch);
+  bool dead = false;    // a wait of this thread gave up
+  int s = 0;            // ring stage of the next chunk
+  unsigned parity = 0;  // and the parity of its phase
+  StgStep cur = stg_step<MODE>(O, 0, k, R, C, NG, g);
   for (int i = 0; i < C; ++i) {
-    const int c = MODE == 0 ? i : C - 1 - i;
-    const int r0 = __ldg(L.RS + c * (R + 1) + k), r1 = __ldg(L.RS + c * (R + 1) + k + 1);
-    if (r0 < r1) {
-      const int step = c * R + k;
-      // this group's rows: srow[j0 .. j1)
-      int j = r0 + __ldg(O.goff + (long long)step * (NG + 1) + g);
-      const int j1 = r0 + __ldg(O.goff + (long long)step * (NG + 1) + g + 1);
+    const StgStep nxt = stg_step<MODE>(O, i + 1, k, R, C, NG, g);
+    if (cur.h.y > 0) {
       // the current row, the next (its diagonal inverse and b in flight) and
       // the one after (its index in flight)
-      int row = j < j1 ? __ldg(O.srow + j) : -1;
-      int rown = j + 1 < j1 ? __ldg(O.srow + j + 1) : -1;
-      int rown2 = j + 2 < j1 ? __ldg(O.srow + j + 2) : -1;
+      int row = cur.g.x, rown = cur.g.y, j2 = cur.g.z;
+      const int j1 = cur.g.w;
+      int rown2 = j2 < j1 ? __ldg(O.srow + j2) : -1;
       V di[D], bv[D], dn[D], bn[D];
       stg_row_data<D, V>(L, row, row >= 0 && lane < D, lane, di, bv);
       stg_row_data<D, V>(L, rown, rown >= 0 && lane < D, lane, dn, bn);
-      if (i > 0 && !wait_regions<STG_T>(L.nb + nb0, nnb, pg, epoch, (unsigned)i, abort_flag)) break;
-      const int nact = __ldg(O.step_nact + step), ne = EPT * nact;
-      const long long nch = (__ldg(O.step_off + step + 1) - __ldg(O.step_off + step)) / ne;
+      const int nact = cur.h.x, ne = EPT * nact;
       V acc[D];
 #pragma unroll
       for (int a = 0; a < D; ++a) acc[a] = V(0);
-      for (long long t = 0; t < nch; ++t, ++q) {
-        const int s = (int)(q % NS);
+      for (int t = 0; t < cur.h.y; ++t) {
         // a wait that gave up leaves the chunk unread by the whole warp, so a
         // lane group never splits between taking and skipping it
-        const bool ok = __all_sync(0xffffffffu, mbar_wait(&full[s], (unsigned)((q / NS) & 1), abort_flag));
+        const bool ok = __all_sync(0xffffffffu, mbar_wait(&full[s], parity, abort_flag));
         const unsigned char* chunk = ring + s * CB;
         int v[EPT];
-        V xj[EPT][D];
+        unsigned u[EPT][W][4];
+        unsigned tagged = 0;  // slots that wait for a new value
 #pragma unroll
         for (int h = 0; h < EPT; ++h) {
           v[h] = ok && tid < nact ? reinterpret_cast<const int*>(chunk)[h * nact + tid] : -1;
           const int col = v[h] & STG_NONE;
-          if (v[h] >= 0 && col != STG_NONE)
-            ldx_vertex<D, false, false, true>((const V*)L.x + (long long)col * D, xj[h]);
+          if (v[h] < 0 || col == STG_NONE) continue;
+          if (MODE == 0 || (v[h] & STG_NEW)) {
+            tagged |= 1u << h;
+#pragma unroll
+            for (int w = 0; w < W; ++w) ld_word(L.xt + (long long)col * W + w, u[h][w]);
+          } else {
+            plain_words((const V*)L.x + (long long)col * D, tag, u[h]);
+          }
         }
+        if constexpr (AT_ONCE) wait_words<EPT, W>(L.xt, v, tagged, tag, u, abort_flag, dead);
 #pragma unroll
         for (int h = 0; h < EPT; ++h) {
           if (v[h] < 0) continue;
-          if ((v[h] & STG_NONE) != STG_NONE) {
+          const int col = v[h] & STG_NONE;
+          if (col != STG_NONE) {
+            if constexpr (!AT_ONCE) {
+#pragma unroll
+              for (int w = 0; w < W; ++w) wait_word(L.xt + (long long)col * W + w, tag, u[h][w], abort_flag, dead);
+            }
+            V xj[D];
+            tagged_values(u[h], xj);
             V blk[9];
             stg_block<V, S>(chunk, ne, h * nact + tid, blk);
 #pragma unroll
             for (int a = 0; a < D; ++a)
 #pragma unroll
-              for (int bb = 0; bb < D; ++bb) acc[a] += blk[a * D + bb] * xj[h][bb];
+              for (int bb = 0; bb < D; ++bb) acc[a] += blk[a * D + bb] * xj[bb];
           }
           if (v[h] & STG_END) {
             // the row is done: the group's sum, x_row, the next row
@@ -1035,34 +1194,38 @@ __device__ __forceinline__ void stg_consume(const LV<V>& L, const StagedOp<S>& O
             for (int o = G / 2; o > 0; o >>= 1)
 #pragma unroll
               for (int a = 0; a < D; ++a) acc[a] += __shfl_xor_sync(gmask, acc[a], o, G);
+            V sum = V(0);
             if (row >= 0 && lane < D) {
-              V sum = V(0);
 #pragma unroll
               for (int bb = 0; bb < D; ++bb) sum += di[bb] * (bv[bb] - acc[bb]);
-              stx<false>(L.x + (long long)row * D + lane, sum);
+            }
+            const V s1 = __shfl_sync(gmask, sum, 1, G), s2 = __shfl_sync(gmask, sum, 2, G);
+            if (row >= 0) {
+              if (lane == 0) st_tagged(L.xt + (long long)row * W, sum, s1, s2, tag);
+              if (lane < D) stx<false>(L.x + (long long)row * D + lane, sum);
             }
 #pragma unroll
             for (int a = 0; a < D; ++a) acc[a] = V(0);
-            ++j;
             row = rown;
             rown = rown2;
 #pragma unroll
             for (int bb = 0; bb < D; ++bb) di[bb] = dn[bb], bv[bb] = bn[bb];
             stg_row_data<D, V>(L, rown, rown >= 0 && lane < D, lane, dn, bn);
-            rown2 = j + 2 < j1 ? __ldg(O.srow + j + 2) : -1;
+            ++j2;
+            rown2 = j2 < j1 ? __ldg(O.srow + j2) : -1;
           }
         }
         __syncwarp();
         if ((tid & 31) == 0) mbar_arrive(&empty[s]);
+        if (++s == NS) s = 0, parity ^= 1u;
       }
     }
-    publish_stage<STG_T>(pg + k, epoch, (unsigned)(i + 1));
+    cur = nxt;
   }
 }
 
 // Forward sweep from zero (MODE 0, lower part) or backward sweep (MODE 1,
-// whole rows) of a 3D region level with the staged operator: the waits and
-// stages of vdown_kernel / vup_kernel.
+// whole rows) of a 3D region level with the staged operator.
 template <int D, int G, typename V, typename S, int MODE>
 __global__ void __launch_bounds__(STG_T + 32, 2)
     vstaged_kernel(const __grid_constant__ LV<V> L, const __grid_constant__ StagedOp<S> O, Scalars* sc) {
@@ -1098,7 +1261,7 @@ template <typename S>
 __global__ void stage_fill_kernel(const int* __restrict__ rp, const int* __restrict__ ci, const S* __restrict__ off,
                                   long long n, const int* __restrict__ RS, int R, int C,
                                   const long long* __restrict__ step_off, const int* __restrict__ step_nact,
-                                  const int* __restrict__ goff, const int* __restrict__ srow, int G,
+                                  const int* __restrict__ goff, const int* __restrict__ srow, int G, int mode,
                                   int* __restrict__ sci, S* __restrict__ sv8, S* __restrict__ sv9) {
   constexpr int EPT = stg_ept<S>();
   const int NG = STG_T / G;
@@ -1127,7 +1290,9 @@ __global__ void stage_fill_kernel(const int* __restrict__ rp, const int* __restr
       for (int t = 0; t < steps; ++t) {
         const int e = t * G + lane;
         const int end = t == steps - 1 ? STG_END : 0;
-        if (e < len) put(ci[a0 + e] | end, a0 + e);
+        // the forward sweep reads earlier colours only; the backward sweep has
+        // written a column when its colour, so its solve index, is the later one
+        if (e < len) put(ci[a0 + e] | end | (mode == 0 || ci[a0 + e] > row ? STG_NEW : 0), a0 + e);
         else put(STG_NONE | end, -1);
       }
     }

@@ -298,158 +298,197 @@ __global__ void __launch_bounds__(256) prolongm_kernel(const __grid_constant__ L
 
 // ------------------------------------------------------------------ staged region sweeps (3D), KR right-hand sides
 
+// A row's KR x D sums over its G lanes (G >= 4), each value summed over the
+// xor tree of rowm_finish.  While more than one right-hand side is left, a lane
+// passes half of its sums on and keeps the other half, so a row of 8
+// right-hand sides and 32 lanes takes 27 shuffles and not 120, and each lane
+// ends with one right-hand side's D sums in acc[0] (two, in acc[0] and acc[1],
+// for 8 right-hand sides on 4 lanes).  Every value is the sum of the same
+// pairs, so its bits are those of the full exchange.
+template <int D, int KR, typename V>
+__device__ __forceinline__ void row_sums_split(V (&acc)[KR][D], int lane, int G, unsigned gmask) {
+  int o = G / 2;
+#pragma unroll
+  for (int m = KR / 2; m > 0; m /= 2) {
+    if (o == 0) break;
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int r = 0; r < m; ++r)
+#pragma unroll
+      for (int a = 0; a < D; ++a) {
+        const V give = up ? acc[r][a] : acc[r + m][a], keep = up ? acc[r + m][a] : acc[r][a];
+        acc[r][a] = keep + __shfl_xor_sync(gmask, give, o, G);
+      }
+    o >>= 1;
+  }
+  for (; o > 0; o >>= 1)
+#pragma unroll
+    for (int a = 0; a < D; ++a) acc[0][a] += __shfl_xor_sync(gmask, acc[0][a], o, G);
+}
+
+// Up to 4 right-hand sides the multi sweeps wait for tagged values as the
+// single ones do, word r of a vertex for right-hand side r; with 8 a slot's
+// words take 32 registers and every one of its 8 loads goes to L2, and the
+// regions' stage waits, with their gathers through L1, are faster.  56^3 graded
+// BF16, V-cycle, stage waits against tags: k = 2 3677 and 2517 us, k = 4 3849
+// and 3174 us, k = 8 4915 and 5616 us.
+constexpr bool stgm_tags(int KR) { return KR <= 4; }
+
 // The consumers of vstaged_kernel with KR right-hand sides: the same chunks of
 // the level's staged copy (the producer is stg_produce), each slot applied to
 // the KR interleaved vectors of its column, each right-hand side's sums in the
-// order of rowm_finish.  b of a row is loaded when its group starts the row.
+// order of rowm_finish.  D^-1 and b of a row are loaded when its group starts
+// the row; a lane holds b of the right-hand sides whose sums it ends with.
 template <int D, int KR, typename V, typename S, int MODE>
 __device__ __forceinline__ void stgm_consume(const LV<V>& L, const StagedOp<S>& O, int k, int R, int C,
                                              unsigned epoch, unsigned long long* full, unsigned long long* empty,
                                              const unsigned char* ring, int* abort_flag, int G) {
   constexpr int NS = stg_stages<S>(), CB = stg_chunk_bytes<S>(), EPT = stg_ept<S>(), N = KR * D;
+  constexpr int NL = KR == 8 ? 2 : 1;  // right-hand sides a lane may end with
+  constexpr bool TAGS = stgm_tags(KR);
+  constexpr int PK = KR > 4 ? 1 : 2;   // slots whose gathers are in flight together
+  // all words of PK slots waited for together (k = 4: V-cycle 3174 us, slot by
+  // slot 3559), or slot by slot (k = 2: 2517 us, together 2690)
+  constexpr bool AT_ONCE = KR == 4;
   const int NG = STG_T / G;
   const int tid = threadIdx.x, g = tid / G, lane = tid & (G - 1);
   const unsigned gmask = G == 32 ? 0xffffffffu : (((1u << G) - 1u) << ((tid & 31) & ~(G - 1)));
+  const unsigned tag = sweep_tag<MODE>(epoch);
+  bool dead = false;  // a wait of this thread gave up
   const int nb0 = __ldg(L.nb_rp + k), nnb = __ldg(L.nb_rp + k + 1) - nb0;
   unsigned long long* pg = MODE == 0 ? L.pg_d : L.pg_u;
-  long long q = 0;  // chunks taken
+  const int sub = G / KR;  // lanes that end with the same right-hand side (0: a lane has two)
+  // the right-hand side row_sums_split leaves this lane (the lane's top bits)
+  const int rl = sub > 0 ? lane / sub : 2 * lane;
+  const int sl = sub > 0 ? lane - rl * sub : 0;
+  int s = 0;            // ring stage of the next chunk
+  unsigned parity = 0;  // and the parity of its phase
+  StgStep cur = stg_step<MODE>(O, 0, k, R, C, NG, g);
   for (int i = 0; i < C; ++i) {
-    const int c = MODE == 0 ? i : C - 1 - i;
-    const int r0 = __ldg(L.RS + c * (R + 1) + k), r1 = __ldg(L.RS + c * (R + 1) + k + 1);
-    if (r0 < r1) {
-      const int step = c * R + k;
-      int j = r0 + __ldg(O.goff + (long long)step * (NG + 1) + g);
-      const int j1 = r0 + __ldg(O.goff + (long long)step * (NG + 1) + g + 1);
-      int row = j < j1 ? __ldg(O.srow + j) : -1;
-      int rown = j + 1 < j1 ? __ldg(O.srow + j + 1) : -1;
-      V di[D], bv[N];
+    StgStep nxt;
+    if constexpr (KR <= 4) nxt = stg_step<MODE>(O, i + 1, k, R, C, NG, g);
+    if (cur.h.y > 0) {
+      int row = cur.g.x, rown = cur.g.y, j2 = cur.g.z;
+      const int j1 = cur.g.w;
+      V di[D * D], bv[NL][D];
       auto row_data = [&]() {
-        if (row >= 0 && lane < D) {
+        if (row >= 0) {
 #pragma unroll
-          for (int bb = 0; bb < D; ++bb) di[bb] = __ldg((const V*)L.dinv + (long long)(lane * D + bb) * L.nv + row);
-          ld_vec_n<N, false>((const V*)L.b + (long long)row * N, bv);
+          for (int e = 0; e < D * D; ++e) di[e] = __ldg((const V*)L.dinv + (long long)e * L.nv + row);
+#pragma unroll
+          for (int u = 0; u < NL; ++u)
+            if (u == 0 || sub == 0) {
+#pragma unroll
+              for (int a = 0; a < D; ++a) bv[u][a] = ldx<false>((const V*)L.b + (long long)row * N + (rl + u) * D + a);
+            }
         }
       };
       row_data();
-      if (i > 0 && !wait_regions<STG_T>(L.nb + nb0, nnb, pg, epoch, (unsigned)i, abort_flag)) break;
-      const int nact = __ldg(O.step_nact + step), ne = EPT * nact;
-      const long long nch = (__ldg(O.step_off + step + 1) - __ldg(O.step_off + step)) / ne;
+      if constexpr (!TAGS) {
+        if (i > 0 && !wait_regions<STG_T>(L.nb + nb0, nnb, pg, epoch, (unsigned)i, abort_flag)) break;
+      }
+      const int nact = cur.h.x, ne = EPT * nact;
       V acc[KR][D];
 #pragma unroll
       for (int r = 0; r < KR; ++r)
 #pragma unroll
         for (int a = 0; a < D; ++a) acc[r][a] = V(0);
-      for (long long t = 0; t < nch; ++t, ++q) {
-        const int s = (int)(q % NS);
+      for (int t = 0; t < cur.h.y; ++t) {
         // warp-uniform: a lane group never splits between taking and skipping a chunk
-        const bool ok = __all_sync(0xffffffffu, mbar_wait(&full[s], (unsigned)((q / NS) & 1), abort_flag));
+        const bool ok = __all_sync(0xffffffffu, mbar_wait(&full[s], parity, abort_flag));
         const unsigned char* chunk = ring + s * CB;
-        // up to 4 right-hand sides, two slots at a time with their gathers in
-        // flight together; 8 right-hand sides one slot at a time (registers)
-        if constexpr (KR > 4) {
-#pragma unroll
-        for (int h = 0; h < EPT; ++h) {
-          const int v = ok && tid < nact ? reinterpret_cast<const int*>(chunk)[h * nact + tid] : -1;
-          if (v < 0) continue;
-          const int col = v & STG_NONE;
-          if (col != STG_NONE) {
-            V xj[N];
-            ld_vec_n<N, true>((const V*)L.x + (long long)col * N, xj);
-            V blk[9];
-            stg_block<V, S>(chunk, ne, h * nact + tid, blk);
-#pragma unroll
-            for (int r = 0; r < KR; ++r)
-#pragma unroll
-              for (int a = 0; a < D; ++a)
-#pragma unroll
-                for (int bb = 0; bb < D; ++bb) acc[r][a] += blk[a * D + bb] * xj[r * D + bb];
-          }
-          if (v & STG_END) {
-            // the row is done: the group's sums, x_row of every right-hand side, the next row
-            for (int o = G / 2; o > 0; o >>= 1)
-#pragma unroll
-              for (int r = 0; r < KR; ++r)
-#pragma unroll
-                for (int a = 0; a < D; ++a) acc[r][a] += __shfl_xor_sync(gmask, acc[r][a], o, G);
-            if (row >= 0 && lane < D) {
-#pragma unroll
-              for (int r = 0; r < KR; ++r) {
-                V sum = V(0);
-#pragma unroll
-                for (int bb = 0; bb < D; ++bb) sum += di[bb] * (bv[r * D + bb] - acc[r][bb]);
-                __stcg((V*)L.x + ((long long)row * KR + r) * D + lane, sum);
-              }
-            }
-#pragma unroll
-            for (int r = 0; r < KR; ++r)
-#pragma unroll
-              for (int a = 0; a < D; ++a) acc[r][a] = V(0);
-            ++j;
-            row = rown;
-            rown = j + 1 < j1 ? __ldg(O.srow + j + 1) : -1;
-            row_data();
-          }
-        }
-        } else {
-        constexpr int PK = 2;
+        // PK slots at a time, their gathers in flight together
 #pragma unroll
         for (int h0 = 0; h0 < EPT; h0 += PK) {
           int vv[PK];
-          V xj[PK][N];
+          unsigned xw[PK][KR][4];  // per right-hand side its D = 3 values (and the tag)
+          unsigned tagged = 0;     // slots that wait for a new value
 #pragma unroll
           for (int u = 0; u < PK; ++u) {
             vv[u] = ok && tid < nact ? reinterpret_cast<const int*>(chunk)[(h0 + u) * nact + tid] : -1;
             const int col = vv[u] & STG_NONE;
-            if (vv[u] >= 0 && col != STG_NONE) ld_vec_n<N, true>((const V*)L.x + (long long)col * N, xj[u]);
-          }
+            if (vv[u] < 0 || col == STG_NONE) continue;
+            if (TAGS && (MODE == 0 || (vv[u] & STG_NEW))) {
+              tagged |= 1u << u;
 #pragma unroll
-          for (int u = 0; u < PK; ++u) {
-          const int v = vv[u], h = h0 + u;
-          if (v < 0) continue;
-          const int col = v & STG_NONE;
-          if (col != STG_NONE) {
-            V blk[9];
-            stg_block<V, S>(chunk, ne, h * nact + tid, blk);
-#pragma unroll
-            for (int r = 0; r < KR; ++r)
-#pragma unroll
-              for (int a = 0; a < D; ++a)
-#pragma unroll
-                for (int bb = 0; bb < D; ++bb) acc[r][a] += blk[a * D + bb] * xj[u][r * D + bb];
-          }
-          if (v & STG_END) {
-            // the row is done: the group's sums, x_row of every right-hand side, the next row
-            for (int o = G / 2; o > 0; o >>= 1)
+              for (int r = 0; r < KR; ++r) ld_word(L.xt + (long long)col * KR + r, xw[u][r]);
+            } else {
+              V xj[N];
+              ld_vec_n<N, true>((const V*)L.x + (long long)col * N, xj);
 #pragma unroll
               for (int r = 0; r < KR; ++r)
 #pragma unroll
-                for (int a = 0; a < D; ++a) acc[r][a] += __shfl_xor_sync(gmask, acc[r][a], o, G);
-            if (row >= 0 && lane < D) {
+                for (int a = 0; a < D; ++a) xw[u][r][a] = __float_as_uint(xj[r * D + a]);
+              if constexpr (TAGS && !AT_ONCE) {
 #pragma unroll
-              for (int r = 0; r < KR; ++r) {
-                V sum = V(0);
-#pragma unroll
-                for (int bb = 0; bb < D; ++bb) sum += di[bb] * (bv[r * D + bb] - acc[r][bb]);
-                __stcg((V*)L.x + ((long long)row * KR + r) * D + lane, sum);
+                for (int r = 0; r < KR; ++r) xw[u][r][3] = tag;
               }
             }
-#pragma unroll
-            for (int r = 0; r < KR; ++r)
-#pragma unroll
-              for (int a = 0; a < D; ++a) acc[r][a] = V(0);
-            ++j;
-            row = rown;
-            rown = j + 1 < j1 ? __ldg(O.srow + j + 1) : -1;
-            row_data();
           }
+          if constexpr (TAGS && AT_ONCE) wait_words<PK, KR>(L.xt, vv, tagged, tag, xw, abort_flag, dead);
+#pragma unroll
+          for (int u = 0; u < PK; ++u) {
+            const int v = vv[u], h = h0 + u;
+            if (v < 0) continue;
+            const int col = v & STG_NONE;
+            if (col != STG_NONE) {
+              V blk[9];
+              stg_block<V, S>(chunk, ne, h * nact + tid, blk);
+#pragma unroll
+              for (int r = 0; r < KR; ++r) {
+                if constexpr (TAGS && !AT_ONCE)
+                  wait_word(L.xt + (long long)col * KR + r, tag, xw[u][r], abort_flag, dead);
+#pragma unroll
+                for (int a = 0; a < D; ++a)
+#pragma unroll
+                  for (int bb = 0; bb < D; ++bb) acc[r][a] += blk[a * D + bb] * __uint_as_float(xw[u][r][bb]);
+              }
+            }
+            if (v & STG_END) {
+              // the row is done: the group's sums, x_row of every right-hand side, the next row
+              row_sums_split<D, KR, V>(acc, lane, G, gmask);
+              if (row >= 0) {
+#pragma unroll
+                for (int w = 0; w < NL; ++w) {
+                  if (w == 1 && sub > 0) break;
+                  V sum[D];
+#pragma unroll
+                  for (int a = 0; a < D; ++a) {
+                    sum[a] = V(0);
+#pragma unroll
+                    for (int bb = 0; bb < D; ++bb) sum[a] += di[a * D + bb] * (bv[w][bb] - acc[w][bb]);
+                  }
+                  // the lanes of a right-hand side share its sums: one writes the tagged word
+                  if (TAGS && sl == 0) st_tagged(L.xt + (long long)row * KR + rl + w, sum[0], sum[1], sum[2], tag);
+                  V* xr = (V*)L.x + ((long long)row * KR + rl + w) * D;
+                  if (sub >= 4) {
+                    if (sl < D) __stcg(xr + sl, pick<D>(sum, sl));
+                  } else if (sl == 0) {
+#pragma unroll
+                    for (int a = 0; a < D; ++a) __stcg(xr + a, sum[a]);
+                  }
+                }
+              }
+#pragma unroll
+              for (int r = 0; r < KR; ++r)
+#pragma unroll
+                for (int a = 0; a < D; ++a) acc[r][a] = V(0);
+              row = rown;
+              rown = j2 < j1 ? __ldg(O.srow + j2) : -1;
+              ++j2;
+              row_data();
+            }
           }
-        }
         }
         __syncwarp();
         if ((tid & 31) == 0) mbar_arrive(&empty[s]);
+        if (++s == NS) s = 0, parity ^= 1u;
       }
     }
-    publish_stage<STG_T>(pg + k, epoch, (unsigned)(i + 1));
+    // (8 right-hand sides have no registers to hold it through the step)
+    if constexpr (KR > 4) nxt = stg_step<MODE>(O, i + 1, k, R, C, NG, g);
+    if constexpr (!TAGS) publish_stage<STG_T>(pg + k, epoch, (unsigned)(i + 1));
+    cur = nxt;
   }
 }
 
@@ -877,6 +916,7 @@ struct MultiEngine : MultiBase {
   using V = float;
   EngineView<V> v;
   int cap = 0;                        // right-hand sides the buffers hold (2, 4 or 8)
+  std::vector<DevBuf<uint4>> xtm;     // 3D region levels: the staged sweeps' tagged values
   std::vector<DevBuf<V>> xm, bm, rm;  // per level, [nv][cap][D] (a pass with KR uses the first nv KR D)
   DevBuf<double> U, r, p, q, Fb, Ub, part, hist;
   DevBuf<Scalars> sc;
@@ -915,6 +955,7 @@ struct MultiEngine : MultiBase {
     }
     cudaStream_t s = v.stream;
     VASMG_CUDA(cudaStreamSynchronize(s));
+    xtm.resize(v.L);
     xm.resize(v.L);
     bm.resize(v.L);
     rm.resize(v.L);
@@ -926,6 +967,12 @@ struct MultiEngine : MultiBase {
       xm[l].zero();
       bm[l].zero();
       rm[l].zero();
+      // a pass with KR takes the first nv KR words; the epochs in the tags go
+      // on from pass to pass and are shared with the single sweeps
+      if (D == 3 && v.lv[l].xt) {
+        xtm[l].alloc(std::max<i64>(1, v.nv[l]) * kr, s);
+        xtm[l].zero();
+      }
     }
     const i64 n = n0();
     U.alloc(n * kr, s);
@@ -953,6 +1000,7 @@ struct MultiEngine : MultiBase {
     a.x = xm[l].get();
     a.b = bm[l].get();
     a.r = rm[l].get();
+    a.xt = xtm[l].get();
     if (l + 1 < v.L) {
       a.bc = bm[l + 1].get();
       a.xc = xm[l + 1].get();
