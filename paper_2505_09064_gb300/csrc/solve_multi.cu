@@ -26,7 +26,6 @@
 namespace vasmg {
 
 constexpr int DFM_THREADS = 256;    // threads of the batched sweep CTAs and of the plain batched kernels
-constexpr int TAILM_THREADS = 512;  // threads of the multi tail CTAs (more registers per thread than the single tail)
 constexpr int KMAX = 8;             // right-hand sides per pass
 constexpr int KG_SPMV = 4;          // right-hand sides per SpMV launch
 
@@ -525,152 +524,34 @@ __global__ void __launch_bounds__(STG_T + 32, 2)
 
 // ------------------------------------------------------------------ tail
 
-// One multicolour sweep of a tail level on the cluster, KR right-hand sides.
-template <int D, int KR, typename V, typename S, int MODE>
-__device__ __forceinline__ void tailm_sweep(const TL<V>& L, int gg, int NG, int lane, int G) {
-  const int C = L.ncol;
-  auto colour = [&](int i) { return MODE == 0 ? i : C - 1 - i; };
-  RowPFM<D, KR, V> cur;
-  {
-    const int c = colour(0), q0 = __ldg(L.cs + c), q1 = __ldg(L.cs + c + 1);
-    rowm_prefetch<D, KR, V, S, MODE>(L, q0 + gg, q0 + gg < q1, lane, cur);
-  }
-  for (int i = 0; i < C; ++i) {
-    const int c = colour(i), r0 = __ldg(L.cs + c), r1 = __ldg(L.cs + c + 1);
-    for (int base = r0; base < r1; base += NG) {
-      RowPFM<D, KR, V> nxt;
-      bool have = false;
-      if (base + NG < r1) {
-        rowm_prefetch<D, KR, V, S, MODE>(L, base + NG + gg, base + NG + gg < r1, lane, nxt);
-        have = true;
-      } else if (i + 1 < C) {
-        const int c2 = colour(i + 1), q0 = __ldg(L.cs + c2), q1 = __ldg(L.cs + c2 + 1);
-        rowm_prefetch<D, KR, V, S, MODE>(L, q0 + gg, q0 + gg < q1, lane, nxt);
-        have = true;
-      }
-      rowm_finish<D, KR, V, S, MODE>(L, base + gg, base + gg < r1, lane, G, cur);
-      if (have) cur = nxt;
-    }
-    cluster_sync_all();
-  }
-}
-
 // Entry t of a level's vector of right-hand side i in the interleaved layout.
 template <int D, int KR>
 __device__ __forceinline__ long long mix(long long t, int i) {
   return ((t / D) * KR + i) * D + (t % D);
 }
 
-// Levels ls..L of the V-cycle on CTA 0 for right-hand side i, with the
-// single solve's code (vectors in shared memory): b_ls of right-hand side i
-// comes in, its x_ls goes out.
-template <int D, int KR, typename V, typename S>
-__device__ void tailm_one_cta(const TailArgs<V>& A, int i) {
-  extern __shared__ __align__(16) unsigned char tail_smem[];
-  V* sm = reinterpret_cast<V*>(tail_smem);
-  const int tid = threadIdx.x, NT = blockDim.x;
-  const int ls = A.ls, Lc = A.L, n_ls = A.lv[ls].nv * D;
-  {
-    const TL<V> Ls = shared_level<D, V>(A, ls, sm);
-    for (int t = tid; t < n_ls; t += NT) Ls.b[t] = __ldcg(A.lv[ls].b + mix<D, KR>(t, i));
-  }
-  __syncthreads();
-  one_cta_down<D, V, S>(A, sm, ls, Lc);
-  {
-    const TL<V> Lcs = shared_level<D, V>(A, Lc, sm);
-    if (threadIdx.x < 32) coarse_solve_warp<V, true>(A.co, Lcs.b, Lcs.x);
-  }
-  __syncthreads();
-  one_cta_up<D, V, S>(A, sm, Lc, ls);
-  {
-    const TL<V> Ls = shared_level<D, V>(A, ls, sm);
-    for (int t = tid; t < n_ls; t += NT) __stcg(A.lv[ls].x + mix<D, KR>(t, i), Ls.x[t]);
-  }
-  __syncthreads();
-}
-
-// x_kd = M b_kd for every right-hand side on every CTA of the cluster: b_kd of
-// each right-hand side staged in shared memory (zero-padded to the row
-// stride), one warp per row of M; every right-hand side's sums are formed as
-// in dense_level_rows.
-template <int D, int KR>
-__device__ __forceinline__ void dense_rows_m(const TailArgs<float>& A, float* sb, int rank, int nct) {
-  const int n = A.dn, ld = A.dld, ld4 = ld >> 2;
-  const float* b = A.lv[A.kd].b;
-  float* x = A.lv[A.kd].x;
-  for (int t = threadIdx.x; t < KR * ld; t += blockDim.x) {
-    const int i = t / ld, c = t - i * ld;
-    sb[t] = c < n ? __ldcg(b + mix<D, KR>(c, i)) : 0.0f;
-  }
-  __syncthreads();
-  const float4* sb4 = reinterpret_cast<const float4*>(sb);
-  const int wpc = blockDim.x >> 5, lane = threadIdx.x & 31;
-  const int nw = nct * wpc;
-  for (int t = rank * wpc + ((int)threadIdx.x >> 5); t < n; t += nw) {
-    const float4* m4 = reinterpret_cast<const float4*>(A.dm + (long long)t * ld);
-    float a[KR][4];
-#pragma unroll
-    for (int i = 0; i < KR; ++i) a[i][0] = a[i][1] = a[i][2] = a[i][3] = 0.0f;
-    for (int j = lane; j < ld4; j += 32) {
-      const float4 mv = __ldg(m4 + j);
-#pragma unroll
-      for (int i = 0; i < KR; ++i) {
-        const float4 bv = sb4[i * ld4 + j];
-        a[i][0] += mv.x * bv.x;
-        a[i][1] += mv.y * bv.y;
-        a[i][2] += mv.z * bv.z;
-        a[i][3] += mv.w * bv.w;
-      }
-    }
-#pragma unroll
-    for (int i = 0; i < KR; ++i) {
-      float acc = (a[i][0] + a[i][1]) + (a[i][2] + a[i][3]);
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-      if (lane == 0) __stcg(x + mix<D, KR>(t, i), acc);
-    }
-  }
-}
-
-// The V-cycle of the small levels for KR right-hand sides: the cluster levels
-// with all of them at once, the one-CTA levels one right-hand side at a time,
-// the dense level for all at once.
-template <int D, int KR, typename S>
-__global__ void __launch_bounds__(TAILM_THREADS) tailm_kernel(const __grid_constant__ TailArgs<float> A) {
-  extern __shared__ __align__(16) unsigned char tail_smem[];
-  using V = float;
-  constexpr int G = tail_g<D>();
-  const int nct = (int)cluster_size(), rank = (int)cluster_rank();
-  // rows dealt to the CTAs first, then to their warps (as tail_run)
-  const int NG = nct * ((int)blockDim.x / G);
-  const int gg = (((int)threadIdx.x >> 5) * nct + rank) * (32 / G) + ((int)threadIdx.x & 31) / G;
-  const int lane = threadIdx.x & (G - 1);
-  const int tid = rank * blockDim.x + threadIdx.x, NT = nct * blockDim.x;
-  const int l0 = A.l0, ls = A.ls;
-  for (int l = l0; l < ls; ++l) {
-    const TL<V>& L = A.lv[l];
-    tailm_sweep<D, KR, V, S, 0>(L, gg, NG, lane, G);
-    for (int base = 0; base < L.nv; base += NG) {
-      RowPFM<D, KR, V> st;
-      rowm_prefetch<D, KR, V, S, 2>(L, base + gg, base + gg < L.nv, lane, st);
-      rowm_finish<D, KR, V, S, 2>(L, base + gg, base + gg < L.nv, lane, G, st);
-    }
-    cluster_sync_all();
-    for (int I = tid; I < L.nvc; I += NT) restrictm_row<D, KR, V>(L, I);
-    cluster_sync_all();
-  }
-  if (A.kd >= 0) {
-    dense_rows_m<D, KR>(A, reinterpret_cast<float*>(tail_smem) + A.dsoff, rank, nct);
-  } else if (rank == 0) {
-    for (int i = 0; i < KR; ++i) tailm_one_cta<D, KR, V, S>(A, i);
-  }
+// The V-cycle of the small levels for KR right-hand sides: cluster i of the
+// launch runs the single solve's tail (tail_run) for right-hand side i, on
+// vectors of its own; b of the first tail level comes in from the interleaved
+// vectors and its x goes back to them.  These levels are bound by the latency
+// of their colour steps, and their operators stay in L2, so the clusters run
+// side by side at the single tail's time: k = 8 in 3D (4913 vertices) 471 ->
+// 160 us, k = 4 in 2D (16,641 vertices) 225 -> 99 us against one cluster for
+// all right-hand sides.
+template <int D, typename S>
+__global__ void __launch_bounds__(tail_threads<D, float>(), 1)
+    tailm_kernel(const TailArgs<float>* __restrict__ args, const float* b, float* x, int KR) {
+  const int nct = (int)cluster_size();
+  const int i = (int)blockIdx.x / nct;
+  const TailArgs<float>& A = args[i];
+  const TL<float>& L = A.lv[A.l0];
+  const int n = L.nv * D, NT = nct * (int)blockDim.x;
+  const int tid = (int)cluster_rank() * (int)blockDim.x + (int)threadIdx.x;
+  auto mix = [&](int t) { return ((long long)(t / D) * KR + i) * D + t % D; };
+  for (int t = tid; t < n; t += NT) __stcg(L.b + t, __ldcg(b + mix(t)));
   cluster_sync_all();
-  for (int l = ls - 1; l >= l0; --l) {
-    const TL<V>& L = A.lv[l];
-    for (int i = tid; i < L.nv; i += NT) prolongm_row<D, KR, V>(L, i);
-    cluster_sync_all();
-    tailm_sweep<D, KR, V, S, 1>(L, gg, NG, lane, G);
-  }
+  tail_run<D, float, S>(A);
+  for (int t = tid; t < n; t += NT) __stcg(x + mix(t), __ldcg((const float*)L.x + t));
 }
 
 // ------------------------------------------------------------------ outer CG, KR right-hand sides (FP64)
@@ -917,6 +798,10 @@ struct MultiEngine : MultiBase {
   EngineView<V> v;
   int cap = 0;                        // right-hand sides the buffers hold (2, 4 or 8)
   std::vector<DevBuf<uint4>> xtm;     // 3D region levels: the staged sweeps' tagged values
+  // the tail's vectors and arguments of every right-hand side
+  DevBuf<V> tvec;
+  DevBuf<double> ty;
+  DevBuf<TailArgs<V>> targs;
   std::vector<DevBuf<V>> xm, bm, rm;  // per level, [nv][cap][D] (a pass with KR uses the first nv KR D)
   DevBuf<double> U, r, p, q, Fb, Ub, part, hist;
   DevBuf<Scalars> sc;
@@ -989,6 +874,7 @@ struct MultiEngine : MultiBase {
     sc.zero();
     ctl.alloc(2, s);
     ctl.zero();
+    build_tail(kr);
     if (!host_sc) VASMG_CUDA(cudaMallocHost((void**)&host_sc, sizeof(Scalars) * KMAX));
     if (!host_ctl) VASMG_CUDA(cudaMallocHost((void**)&host_ctl, sizeof(int) * 2));
     cap = kr;
@@ -1126,40 +1012,92 @@ struct MultiEngine : MultiBase {
     }
     if ((phases & 2) && !sweep_staged<KR, 1>(l, a, s)) coop(vupm_kernel<D, KR, V, S>, a.R, a, v.G[l], s);
   }
-  template <int KR>
-  size_t tail_smem_bytes() const {
-    size_t smem = v.tail_smem_base;
-    if (v.ta.kd >= 0) smem = (size_t)v.ta.dsoff * sizeof(V) + sizeof(V) * (size_t)KR * v.ta.dld;
-    return smem;
-  }
-  template <int KR>
-  void tail(cudaStream_t s) {
-    TailArgs<V> ta = v.ta;
-    for (int l = 0; l < v.L; ++l) {
-      ta.lv[l].x = xm[l].get();
-      ta.lv[l].b = bm[l].get();
-      ta.lv[l].r = rm[l].get();
-      if (l + 1 < v.L) {
-        ta.lv[l].bc = bm[l + 1].get();
-        ta.lv[l].xc = xm[l + 1].get();
-      }
+  // Every right-hand side's tail vectors and arguments, for passes of up to kr.
+  void build_tail(int kr) {
+    cudaStream_t s = v.stream;
+    const int l0 = v.lt;
+    i64 words = 0;
+    // a vector starts on a 256-byte boundary
+    auto take = [&](i64 n) {
+      const i64 at = words;
+      words += ceil_div(std::max<i64>(1, n), 64) * 64;
+      return at;
+    };
+    std::vector<i64> at(v.L * 4);
+    for (int l = l0; l < v.L; ++l) {
+      for (int q = 0; q < 3; ++q) at[l * 4 + q] = take(v.nv[l] * D);
+      at[l * 4 + 3] = v.ta.lv[l].xoff >= 0 ? take(v.nv[l] * xs_stride<D, V>() + 4) : -1;
     }
-    const size_t smem = tail_smem_bytes<KR>();
-    VASMG_CHECK(smem <= (size_t)TAIL_SMEM_MAX, VASMG_ERR_UNSUPPORTED,
-                "tail levels too large for shared memory with this many right-hand sides");
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(v.nct);
-    cfg.blockDim = dim3(TAILM_THREADS);
-    cfg.dynamicSmemBytes = smem;
+    tvec.alloc(words * kr, s);
+    tvec.zero();
+    ty.alloc(std::max<i64>(1, (i64)v.ta.co.n) * kr, s);
+    std::vector<TailArgs<V>> ta(kr, v.ta);
+    for (int i = 0; i < kr; ++i) {
+      V* base = tvec.get() + words * i;
+      for (int l = l0; l < v.L; ++l) {
+        TL<V>& t = ta[i].lv[l];
+        t.x = base + at[l * 4];
+        t.b = base + at[l * 4 + 1];
+        t.r = base + at[l * 4 + 2];
+        if (t.xoff >= 0) t.xg = base + at[l * 4 + 3];
+        if (l + 1 < v.L) {
+          t.xc = base + at[(l + 1) * 4];
+          t.bc = base + at[(l + 1) * 4 + 1];
+        }
+      }
+      ta[i].co.y = ty.get() + (i64)std::max(1, v.ta.co.n) * i;
+      ta[i].abort = &sc.get()->abort;
+    }
+    targs.alloc(kr, s);
+    targs.upload(ta.data(), kr);
+  }
+  // CTAs per cluster: the single tail's, or fewer where the device cannot hold
+  // a cluster for every right-hand side at once (no value depends on it): 7
+  // clusters of 16 CTAs fit a GB300 and 8 of 12, so k = 8 takes 12 (160 us in
+  // 3D; 222 with 8)
+  int tail_nct[4] = {0, 0, 0, 0};
+  template <int KR>
+  int tail_cluster() {
+    int& nct = tail_nct[slot(KR)];
+    if (nct) return nct;
+    VASMG_CUDA(cudaFuncSetAttribute(tailm_kernel<D, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, TAIL_SMEM_MAX));
+    nct = v.nct;
+    if (nct > 8)
+      VASMG_CUDA(cudaFuncSetAttribute(tailm_kernel<D, S>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    for (; nct > 4; nct -= 2) {
+      cudaLaunchConfig_t cfg;
+      cudaLaunchAttribute at[1];
+      tail_config(cfg, at, nct, KR, 0);
+      int held = 0;
+      const cudaError_t e = cudaOccupancyMaxActiveClusters(&held, tailm_kernel<D, S>, &cfg);
+      if (e == cudaSuccess && held >= KR) break;
+      cudaGetLastError();
+    }
+    return nct;
+  }
+  void tail_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* at, int nct, int KR, cudaStream_t s) const {
+    cfg = cudaLaunchConfig_t{};
+    cfg.gridDim = dim3(nct * KR);
+    cfg.blockDim = dim3(tail_threads<D, V>());
+    cfg.dynamicSmemBytes = v.tail_smem;
     cfg.stream = s;
-    cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = v.nct;
+    at[0].val.clusterDim.x = nct;
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    VASMG_CUDA(cudaLaunchKernelEx(&cfg, tailm_kernel<D, KR, S>, ta));
+  }
+  template <int KR>
+  void tail(cudaStream_t s) {
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute at[1];
+    tail_config(cfg, at, tail_cluster<KR>(), KR, s);
+    const TailArgs<V>* ta = targs.get();
+    const float* b = bm[v.lt].get();
+    float* x = xm[v.lt].get();
+    const int kr = KR;
+    VASMG_CUDA(cudaLaunchKernelEx(&cfg, tailm_kernel<D, S>, ta, b, x, kr));
     ++launch_counter;
   }
   template <int KR>
@@ -1191,9 +1129,7 @@ struct MultiEngine : MultiBase {
 
   template <int KR>
   void set_attributes() {
-    VASMG_CUDA(cudaFuncSetAttribute(tailm_kernel<D, KR, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, TAIL_SMEM_MAX));
-    if (v.nct > 8)
-      VASMG_CUDA(cudaFuncSetAttribute(tailm_kernel<D, KR, S>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    tail_cluster<KR>();
     // every region of a level must be resident at once: the multi sweep CTAs
     // must fit as many per SM as the single sweeps' regions need
     int bd = 0, bu = 0;
