@@ -2029,8 +2029,10 @@ __global__ void __launch_bounds__(tail_threads<D, V>(), 1) tail_kernel(const __g
 // The dense level's matrix, column by column: CTA j runs the one-CTA V-cycle
 // from level kd (= A.ls) on the unit vector e_j, with its own coarse-solve
 // scratch, and writes the result to column j of M (row-major, n x n).
+// Two CTAs per SM: a column is a chain of colour steps that leaves an SM mostly
+// idle (33^3 FP32, 2187 columns: update 12.4 -> 11.6 ms).
 template <int D, typename V, typename S>
-__global__ void __launch_bounds__(tail_threads<D, V>(), 1) dense_level_kernel(const __grid_constant__ TailArgs<V> A, V* M,
+__global__ void __launch_bounds__(tail_threads<D, V>(), 2) dense_level_kernel(const __grid_constant__ TailArgs<V> A, V* M,
                                                                    double* yscratch) {
   extern __shared__ __align__(16) unsigned char tail_smem[];
   V* sm = reinterpret_cast<V*>(tail_smem);
