@@ -1,6 +1,7 @@
 // Internal declarations shared by the CUDA sources of libvasmg.
 #pragma once
 
+#include <initializer_list>
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
 #include <stdint.h>
@@ -111,6 +112,14 @@ void scan_exclusive_i32(const int32_t* in, int32_t* out, i64 n, cudaStream_t s);
 // Stable LSD radix sort of u64 keys (low `bits` bits significant), optional
 // int32 payload, in place.
 void radix_sort(u64* keys, int32_t* vals, i64 n, int bits, cudaStream_t s);
+// The same by the bits of the given ranges only, least significant first: a
+// pass per 8 bits.  For pairs (high word << 32 | low word) whose words have few
+// bits, and for keys that come in the order of the bits left out.
+struct BitRange {
+  int from, to;
+};
+void radix_sort(u64* keys, int32_t* vals, i64 n, std::initializer_list<BitRange> ranges, cudaStream_t s);
+int bits_for(u64 maxval);  // bits of a number up to maxval, at least 1
 // Compact sorted keys to their distinct values; returns the new count.
 i64 unique_sorted(u64* keys, i64 n, cudaStream_t s);
 // Row pointers of a sorted (row << 32 | col) key array: rp[r] = first key >= r<<32.
@@ -120,7 +129,6 @@ void minmax_f64(const double* x, i64 n, double* mn, double* mx, cudaStream_t s);
 int32_t max_i32(const int32_t* x, i64 n, cudaStream_t s);
 i64 sum_i64(const i64* x, i64 n, cudaStream_t s);
 
-int bits_for(u64 maxval);
 
 // ------------------------------------------------------------------ hierarchy
 

@@ -185,10 +185,113 @@ __global__ void __launch_bounds__(RS_THREADS) rs_scatter_kernel(const u64* __res
   }
 }
 
-void radix_sort(u64* keys, int32_t* vals, i64 n, int bits, cudaStream_t s) {
+// Up to RS_TILE keys: every pass in one CTA, from and to shared memory.  A
+// setup sorts dozens of arrays this small (the coarse levels'), and a pass of
+// the general sort is three launches.
+struct RsShifts {
+  int n;
+  int shift[8];
+};
+constexpr int RS_SMALL_SMEM = RS_TILE * 2 * (8 + 4);
+template <bool HAS_VAL>
+__global__ void __launch_bounds__(RS_THREADS) rs_small_kernel(u64* __restrict__ keys, int32_t* __restrict__ vals, int n,
+                                                              RsShifts passes) {
+  extern __shared__ __align__(16) unsigned char rs_mem[];
+  u64* kin = reinterpret_cast<u64*>(rs_mem);
+  u64* kout = kin + RS_TILE;
+  int32_t* vin = reinterpret_cast<int32_t*>(kout + RS_TILE);
+  int32_t* vout = vin + RS_TILE;
+  __shared__ int wcnt[RS_WARPS][256];
+  __shared__ int wsum[RS_WARPS];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int i = threadIdx.x; i < n; i += RS_THREADS) {
+    kin[i] = keys[i];
+    if (HAS_VAL) vin[i] = vals[i];
+  }
+  // a warp's keys: `rounds` times 32 consecutive ones
+  const int rounds = (n + RS_THREADS - 1) / RS_THREADS, base = warp * rounds * 32;
+  const unsigned lt = (1u << lane) - 1u;
+  for (int p = 0; p < passes.n; ++p) {
+    const int shift = passes.shift[p];
+    for (int k = threadIdx.x; k < RS_WARPS * 256; k += RS_THREADS) (&wcnt[0][0])[k] = 0;
+    __syncthreads();
+    u64 key[RS_ROUNDS];
+    int32_t val[RS_ROUNDS];
+    int dig[RS_ROUNDS], pos[RS_ROUNDS];
+#pragma unroll
+    for (int r = 0; r < RS_ROUNDS; ++r) {
+      dig[r] = 256;
+      if (r >= rounds) continue;  // the same for the whole CTA
+      const int i = base + r * 32 + lane;
+      const bool valid = i < n;
+      key[r] = valid ? kin[i] : 0ull;
+      if (HAS_VAL) val[r] = valid ? vin[i] : 0;
+      const int d = valid ? (int)((key[r] >> shift) & 255u) : 256;
+      const unsigned peers = __match_any_sync(0xffffffffu, d);
+      const int before = d < 256 ? wcnt[warp][d] : 0;
+      __syncwarp();
+      if (valid && lane == __ffs(peers) - 1) wcnt[warp][d] = before + __popc(peers);
+      __syncwarp();
+      dig[r] = d;
+      pos[r] = before + __popc(peers & lt);
+    }
+    __syncthreads();
+    // thread = digit: its count, the digits before it, the warps before
+    int total = 0;
+#pragma unroll
+    for (int w = 0; w < RS_WARPS; ++w) total += wcnt[w][threadIdx.x];
+    int incl = total;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int up = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += up;
+    }
+    if (lane == 31) wsum[warp] = incl;
+    __syncthreads();
+    int run = incl - total;
+    for (int w = 0; w < warp; ++w) run += wsum[w];
+#pragma unroll
+    for (int w = 0; w < RS_WARPS; ++w) {
+      const int c = wcnt[w][threadIdx.x];
+      wcnt[w][threadIdx.x] = run;
+      run += c;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < RS_ROUNDS; ++r) {
+      if (dig[r] < 256) {
+        const int o = wcnt[warp][dig[r]] + pos[r];
+        kout[o] = key[r];
+        if (HAS_VAL) vout[o] = val[r];
+      }
+    }
+    __syncthreads();
+    u64* tk = kin;
+    kin = kout, kout = tk;
+    int32_t* tv = vin;
+    vin = vout, vout = tv;
+  }
+  for (int i = threadIdx.x; i < n; i += RS_THREADS) {
+    keys[i] = kin[i];
+    if (HAS_VAL) vals[i] = vin[i];
+  }
+}
+
+void radix_sort(u64* keys, int32_t* vals, i64 n, std::initializer_list<BitRange> ranges, cudaStream_t s) {
   if (n <= 1) return;
-  if (bits <= 0) bits = 1;
-  const int passes = (bits + 7) / 8;
+  RsShifts ps{};
+  for (const BitRange& r : ranges)
+    for (int shift = r.from; shift < r.to && ps.n < 8; shift += 8) ps.shift[ps.n++] = shift;
+  if (n <= RS_TILE) {
+    auto launch = [&](auto kern) {
+      VASMG_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, RS_SMALL_SMEM));
+      kern<<<1, RS_THREADS, RS_SMALL_SMEM, s>>>(keys, vals, (int)n, ps);
+    };
+    if (vals) launch(rs_small_kernel<true>);
+    else launch(rs_small_kernel<false>);
+    check_launch("rs_small");
+    return;
+  }
   const i64 ntiles = ceil_div(n, RS_TILE);
   DevBuf<u64> kt;
   DevBuf<int32_t> vt;
@@ -200,8 +303,8 @@ void radix_sort(u64* keys, int32_t* vals, i64 n, int bits, cudaStream_t s) {
   u64* kb = kt.get();
   int32_t* va = vals;
   int32_t* vb = vals ? vt.get() : nullptr;
-  for (int p = 0; p < passes; ++p) {
-    const int shift = 8 * p;
+  for (int p = 0; p < ps.n; ++p) {
+    const int shift = ps.shift[p];
     rs_hist_kernel<<<(unsigned)ntiles, RS_THREADS, 0, s>>>(ka, n, shift, counts.get(), ntiles);
     check_launch("rs_hist");
     scan_exclusive<long long>(counts.get(), counts.get(), 256 * ntiles, s);
@@ -218,6 +321,10 @@ void radix_sort(u64* keys, int32_t* vals, i64 n, int bits, cudaStream_t s) {
     VASMG_CUDA(cudaMemcpyAsync(keys, ka, sizeof(u64) * n, cudaMemcpyDeviceToDevice, s));
     if (vals) VASMG_CUDA(cudaMemcpyAsync(vals, va, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice, s));
   }
+}
+
+void radix_sort(u64* keys, int32_t* vals, i64 n, int bits, cudaStream_t s) {
+  radix_sort(keys, vals, n, {BitRange{0, std::max(1, bits)}}, s);
 }
 
 int bits_for(u64 maxval) {

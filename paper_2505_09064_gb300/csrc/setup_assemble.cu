@@ -232,7 +232,8 @@ void setup_assemble(Ctx& c) {
     keys.alloc(m, s);
     pattern_pairs_kernel<<<grid_for(m, 256), 256, 0, s>>>(c.E.get(), c.ne, nl, c.nv, keys.get());
     check_launch("pattern_pairs");
-    radix_sort(keys.get(), nullptr, m, 32 + bits_for((u64)c.nv), s);
+    const int vb = bits_for((u64)c.nv);
+    radix_sort(keys.get(), nullptr, m, {{0, vb}, {32, 32 + vb}}, s);
     const i64 nnz = unique_sorted(keys.get(), m, s);
     VASMG_CHECK(nnz < (i64)INT32_MAX, VASMG_ERR_UNSUPPORTED, "too many blocks for 32-bit indices");
     L0.nnzb = nnz;

@@ -386,7 +386,10 @@ void setup_colour_and_solve_levels(Ctx& c) {
       renum_keys_kernel<<<grid_for(cl.nv, 256), 256, 0, s>>>(cl.colour.get(), l == 0 && mrank.n ? mrank.get() : nullptr,
                                                               cl.nv, keys.get(), sl.perm.get());
       check_launch("renum_keys");
-      radix_sort(keys.get(), sl.perm.get(), cl.nv, 32 + bits_for((u64)cl.ncol), s);
+      // (the keys of levels without a Morton rank come in the low word's order)
+      const bool ranked = l == 0 && mrank.n;
+      radix_sort(keys.get(), sl.perm.get(), cl.nv,
+                 {{0, ranked ? bits_for((u64)cl.nv) : 0}, {32, 32 + bits_for((u64)cl.ncol)}}, s);
       sl.iperm.alloc(cl.nv, s);
       invert_perm_kernel<<<grid_for(cl.nv, 256), 256, 0, s>>>(sl.perm.get(), cl.nv, sl.iperm.get());
       check_launch("invert_perm");
@@ -415,7 +418,8 @@ void setup_colour_and_solve_levels(Ctx& c) {
       offdiag_keys_kernel<<<grid_for(cl.nv, 256), 256, 0, s>>>(cl.rp.get(), cl.ci.get(), cl.nv, sl.iperm.get(),
                                                                 cnt.get(), keys.get(), ent.get());
       check_launch("offdiag_keys");
-      radix_sort(keys.get(), ent.get(), sl.nnz, 32 + bits_for((u64)cl.nv), s);
+      const int vb = bits_for((u64)cl.nv);
+      radix_sort(keys.get(), ent.get(), sl.nnz, {{0, vb}, {32, 32 + vb}}, s);
       sl.rp.alloc(cl.nv + 1, s);
       sl.ci.alloc(sl.nnz, s);
       sl.sp.alloc(cl.nv, s);
@@ -459,7 +463,8 @@ void setup_colour_and_solve_levels(Ctx& c) {
     ent.alloc(cf.pnnz, s);
     r_keys_kernel<<<grid_for(sf.nv, 256), 256, 0, s>>>(sf.prp.get(), sf.pci.get(), sf.nv, keys.get(), ent.get());
     check_launch("r_keys");
-    radix_sort(keys.get(), ent.get(), cf.pnnz, 32 + bits_for((u64)sg.nv), s);
+    // the fine rows (low word) come in ascending order
+    radix_sort(keys.get(), ent.get(), cf.pnnz, {{32, 32 + bits_for((u64)sg.nv)}}, s);
     sf.rrp.alloc(sg.nv + 1, s);
     rowptr_from_pairs(keys.get(), cf.pnnz, sg.nv, sf.rrp.get(), s);
     sf.rci.alloc(cf.pnnz, s);

@@ -302,7 +302,8 @@ void setup_galerkin(Ctx& c, int l) {
   check_launch("gal_pairs");
   diag_pairs_kernel<<<grid_for(g.nv, 256), 256, 0, s>>>(g.nv, keys.get() + m);
   check_launch("diag_pairs");
-  radix_sort(keys.get(), nullptr, m + g.nv, 32 + bits_for((u64)g.nv), s);
+  const int cb = bits_for((u64)g.nv);
+  radix_sort(keys.get(), nullptr, m + g.nv, {{0, cb}, {32, 32 + cb}}, s);
   g.nnzb = unique_sorted(keys.get(), m + g.nv, s);
   VASMG_CHECK(g.nnzb < (i64)INT32_MAX, VASMG_ERR_UNSUPPORTED, "too many blocks for 32-bit indices");
   g.rp.alloc(g.nv + 1, s);
@@ -317,7 +318,8 @@ void setup_galerkin(Ctx& c, int l) {
   transpose_keys_kernel<<<grid_for(f.nv, 256), 256, 0, s>>>(f.prp.get(), f.pci.get(), f.nv, f.r_keys.get(),
                                                              f.r_ent.get());
   check_launch("transpose_keys");
-  radix_sort(f.r_keys.get(), f.r_ent.get(), f.pnnz, 32 + bits_for((u64)g.nv), s);
+  // the fine rows (low word) come in ascending order
+  radix_sort(f.r_keys.get(), f.r_ent.get(), f.pnnz, {{32, 32 + cb}}, s);
   f.r_rp.alloc(g.nv + 1, s);
   rowptr_from_pairs(f.r_keys.get(), f.pnnz, g.nv, f.r_rp.get(), s);
   galerkin_values(c, l);

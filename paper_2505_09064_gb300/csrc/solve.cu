@@ -85,7 +85,7 @@ __global__ void split_parts_kernel(const int* __restrict__ rp, const int* __rest
 __global__ void sell_keys_kernel(const int* __restrict__ rp, int nv, u64* __restrict__ keys, int* __restrict__ vals) {
   for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < nv; r += gridDim.x * blockDim.x) {
     const u64 len = (u64)(rp[r + 1] - rp[r] + 1);  // + diagonal
-    keys[r] = ((u64)(r >> 10) << 40) | ((1023ull - len) << 30) | (u64)(r & 1023);
+    keys[r] = ((u64)(r >> 10) << 40) | ((1023ull - min((unsigned long long)len, 1023ull)) << 30) | (u64)(r & 1023);
     vals[r] = r;
   }
 }
@@ -516,7 +516,8 @@ struct Engine : EngineBase {
     rows.alloc(nv, s);
     sell_keys_kernel<<<grid_for(nv, 256), 256, 0, s>>>(s0.rp.get(), nv, keys.get(), rows.get());
     check_launch("sell_keys");
-    radix_sort(keys.get(), rows.get(), nv, 64, s);
+    // the rows (low bits) come in ascending order
+    radix_sort(keys.get(), rows.get(), nv, {{30, 40 + bits_for((u64)nv >> 10)}}, s);
     const long long nslices = ceil_div(nv, 32);
     sell_w.alloc(nslices, s);
     DevBuf<long long> wb;
