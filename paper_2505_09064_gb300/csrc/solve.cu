@@ -24,10 +24,11 @@
 //   prolong   x_l += P x_{l+1} (masked at dead dofs);
 //   vup       backward sweep (colours in reverse order) with full rows.
 // The two sweeps are cooperative launches with one CTA per region (a range of
-// spatial keys, one contiguous row range per colour).  A region runs its
-// colours in order; before a colour it waits until every neighbouring region
-// has published the stage it reads (64-bit epoch/stage words, release /
-// acquire at GPU scope).  Every wait is bounded; a wait that gives up raises a
+// spatial keys, one contiguous row range per colour).  On 3D levels a row
+// waits for its neighbours' values, which carry the launch's tag (see "values
+// with tags" in solve_dev.cuh).  On 2D levels a region runs its colours in
+// order; before a colour it waits until every neighbouring region has published
+// the stage it reads (64-bit epoch/stage words, release / acquire at GPU scope).  Every wait is bounded; a wait that gives up raises a
 // global abort flag and the solve returns VASMG_ERR_TIMEOUT.  The last CTA to
 // leave a launch advances its epoch.  Residual, restriction and prolongation
 // have no dependencies within themselves and run as plain kernels.  The
@@ -1129,12 +1130,10 @@ struct Engine : EngineBase {
   }
   // The arguments of a tail launch from level l0: the dense level if there is
   // one, else the one-CTA levels, and above them the levels whose x the CTAs
-  // keep in shared memory (the smaller ones first).  *base: the shared memory
-  // before the staging of b_kd; returns all of it.
-  size_t layout_tail(TailArgs<V>& ta, int l0, size_t* base) {
+  // keep in shared memory (the smaller ones first).  Returns the shared memory.
+  size_t layout_tail(TailArgs<V>& ta, int l0) {
     const bool dense = kd >= 0 && kd >= l0;
     size_t smem = fill_tail_args(ta, l0, dense ? kd : one_cta_start(l0), !dense);
-    *base = smem;
     if (dense) {
       ta.kd = kd;
       ta.dn = dn;
@@ -1206,8 +1205,7 @@ struct Engine : EngineBase {
   }
   void tail(int l0, cudaStream_t s) {
     TailArgs<V> ta;
-    size_t base = 0;
-    const size_t smem = layout_tail(ta, l0, &base);
+    const size_t smem = layout_tail(ta, l0);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(nct);
     cfg.blockDim = dim3(tail_threads<D, V>());
@@ -1472,7 +1470,7 @@ struct Engine : EngineBase {
       v.nv.push_back(c->S[l].nv);
       v.pnnz.push_back(l + 1 < L ? (double)c->C[l].pnnz : 0.0);
     }
-    v.tail_smem = layout_tail(v.ta, lt, &v.tail_smem_base);
+    v.tail_smem = layout_tail(v.ta, lt);
     v.cga = cga;
     v.cga.cond = 0;
     v.cg_blocks = cg_blocks;

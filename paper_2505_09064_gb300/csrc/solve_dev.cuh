@@ -2321,7 +2321,6 @@ struct EngineView {
   std::vector<double> pnnz;        // transfer entries of level l -> l+1
   TailArgs<V> ta;                  // the tail launch from level lt (dense level fields set if used)
   size_t tail_smem = 0;            // its dynamic shared memory
-  size_t tail_smem_base = 0;       // the part before the staging of b_kd
   CGArgs cga;                      // level-0 FP64 operator (SELL), permutation, Dirichlet data
   int cg_blocks = 1, spmv_blocks = 1;
   i64 sell_real_entries = 0;

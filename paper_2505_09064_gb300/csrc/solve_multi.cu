@@ -5,9 +5,9 @@
 //
 // Every kernel of an iteration reads the operators once for all KR vectors:
 // the multicolour sweeps and residuals read each block once and apply it to
-// KR gathered vertex vectors, the transfers read each weight once, the dense
-// coarse level reads M once, and the FP64 SpMV reads each block once for up to
-// four vectors.  The V-cycle's vectors are interleaved, entry (vertex v,
+// KR gathered vertex vectors, the transfers read each weight once, and the FP64
+// SpMV reads each block once for up to four vectors.  The small levels, which
+// latency bounds, run in a cluster per right-hand side.  The V-cycle's vectors are interleaved, entry (vertex v,
 // right-hand side i, component a) at (v KR + i) D + a, so one neighbour gather
 // is one contiguous KR D read.  The outer CG's vectors are stored one
 // right-hand side after another.
