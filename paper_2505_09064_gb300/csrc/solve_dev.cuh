@@ -1405,9 +1405,15 @@ struct TailArgs {
   CoarseArgs co;
 };
 
-__device__ __forceinline__ void cluster_sync_all() {
+__device__ __forceinline__ void cluster_arrive() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
   asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+}
+__device__ __forceinline__ void cluster_sync_all() {
+  cluster_arrive();
+  cluster_wait();
 }
 __device__ __forceinline__ unsigned cluster_rank() {
   unsigned r;
@@ -1637,6 +1643,13 @@ struct XBars {
 // takes about as long as a colour's step), and the range of the one after them,
 // so what follows the colour's barrier is the gathers of x, one shuffle sum and
 // the store.  `out`: x is also written to global memory.
+// The backward X_CLUSTER sweep starts from copies that every CTA has just filled
+// for itself (tail_fetch_xs, which arrives at the cluster barrier): no CTA may
+// send into a copy that is still being filled, or the fill would put the old
+// value back over the new one after its bytes were counted.  So the sweep meets
+// the barrier before its first row's gathers, behind the loads of the first
+// rows' entries.  (The forward sweep writes every entry before it is read, and a
+// cluster barrier separates it from the last reads of the copies.)
 template <int D, int G, typename V, typename S, int MODE, int XM>
 __device__ __forceinline__ void tail_sweep(const TL<V>& level, V* xs, int gg, int NG, int lane, const XBars& xb, bool out) {
   constexpr int NPF = tail_npf<D, V>();
@@ -1688,6 +1701,7 @@ __device__ __forceinline__ void tail_sweep(const TL<V>& level, V* xs, int gg, in
   load(cur, range(cur), sa);
   load(nxt, range(nxt), sb);
   RowEnds sg = range(nn);
+  if constexpr (XM == X_CLUSTER && MODE == 1) cluster_wait();
   // the row at `cur`, then the entries of the one two ahead into its registers
   auto step = [&](TailRow<D, V, S, NPF>& st) __attribute__((always_inline)) {
     const int row = cur.base + gg;
@@ -1708,7 +1722,7 @@ __device__ __forceinline__ void tail_sweep(const TL<V>& level, V* xs, int gg, in
       }
     }
     const bool last = nxt.i != cur.i;  // of its colour
-    if (XM == X_GLOBAL && last) asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
+    if (XM == X_GLOBAL && last) cluster_arrive();
     load(nn, sg, st);
     const int done = cur.i;
     cur = nxt;
@@ -1718,7 +1732,7 @@ __device__ __forceinline__ void tail_sweep(const TL<V>& level, V* xs, int gg, in
       sg = range(nn);
     }
     if (last) {
-      if (XM == X_GLOBAL) asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+      if (XM == X_GLOBAL) cluster_wait();
       if (XM == X_CTA) __syncthreads();
       if (XM == X_CLUSTER) mbar_wait(xb.bar + done, xb.parity, xb.abort);
     }
@@ -1819,6 +1833,8 @@ __device__ __forceinline__ void tail_prolong_xs(const TL<V>& L, const V* xs, con
     }
   }
 }
+// Fills this CTA's copy and arrives at the cluster barrier that the backward
+// sweep waits for.
 template <int D, typename V>
 __device__ __forceinline__ void tail_fetch_xs(const TL<V>& L, V* xs) {
   const float4* g = reinterpret_cast<const float4*>(L.xg);
@@ -1826,7 +1842,8 @@ __device__ __forceinline__ void tail_fetch_xs(const TL<V>& L, V* xs) {
   const int n16 = (L.nv * xs_bytes<D, V>() + 15) / 16;  // both copies are padded to 16 bytes
 #pragma unroll 4
   for (int t = threadIdx.x; t < n16; t += blockDim.x) o[t] = __ldcg(g + t);
-  __syncthreads();
+  __syncwarp();
+  cluster_arrive();
 }
 
 // Level l of the one-CTA part with its vectors in shared memory: x, b, r of
