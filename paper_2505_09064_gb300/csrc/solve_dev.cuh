@@ -2029,6 +2029,10 @@ __device__ __forceinline__ void tail_run(const TailArgs<V>& A) {
       tail_sweep<D, G, V, S, 1, X_CLUSTER>(L, sm + L.xoff, gg, NG, lane, xb, l == l0 || A.lv[l - 1].xoff < 0);
       xb.parity ^= 1u;
     } else {
+      // x of a coarser level that was swept in the CTAs' copies comes from global
+      // memory here, where other CTAs wrote it (`out`); the colours' mbarriers
+      // order the copies only
+      if (xsc) cluster_sync_all();
       for (int i = tid; i < L.nv; i += NT) prolong_row<D, V>(L, i);
       cluster_sync_all();
       tail_sweep<D, G, V, S, 1, X_GLOBAL>(L, nullptr, gg, NG, lane, xb, true);

@@ -95,3 +95,11 @@ def test_copies_filled_before_rows_arrive(built, dim, n, precision):
     """Every level of these tails has its x in every CTA's shared memory, filled
     from global memory before each backward sweep sends its rows into it."""
     _solve_under_load(dim, n, precision)
+
+
+@pytest.mark.parametrize("dim,n,precision", [(3, 24, "fp32"), (3, 17, "fp64"), (2, 141, "fp64"), (2, 220, "fp32")])
+def test_level_below_in_the_copies(built, dim, n, precision):
+    """A level of these tails does not fit the CTAs' shared memory and the next
+    coarser one does: the prolongation reads values that other CTAs wrote to
+    global memory during the coarser level's sweep."""
+    _solve_under_load(dim, n, precision)
