@@ -843,23 +843,35 @@ __device__ __forceinline__ void mbar_arrive(unsigned long long* b) {
 __device__ __forceinline__ void mbar_arrive_tx(unsigned long long* b, unsigned bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(b)), "r"(bytes) : "memory");
 }
+// CLUSTER: the data the phase guards come from other CTAs of the cluster, so the
+// test acquires at cluster scope (the default is the CTA's).
+template <bool CLUSTER = false>
 __device__ __forceinline__ bool mbar_test(unsigned long long* b, unsigned parity) {
   unsigned done;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n}\n"
-      : "=r"(done)
-      : "r"(smem_u32(b)), "r"(parity)
-      : "memory");
+  if constexpr (CLUSTER)
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(done)
+        : "r"(smem_u32(b)), "r"(parity)
+        : "memory");
+  else
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(done)
+        : "r"(smem_u32(b)), "r"(parity)
+        : "memory");
   return done != 0;
 }
 // Wait for the phase of the given parity to complete.  Gives up (false)
 // after SPIN_LIMIT polls (after the first 64, 64 ns apart), raising the abort
 // flag, or soon after another wait raised it (read every 256 polls; never
 // when abort_flag is null).
+template <bool CLUSTER = false>
 __device__ __forceinline__ bool mbar_wait(unsigned long long* b, unsigned parity, int* abort_flag) {
 #pragma unroll 1
   for (int spins = 0;; ++spins) {
-    if (mbar_test(b, parity)) return true;
+    if (mbar_test<CLUSTER>(b, parity)) return true;
     if (spins >= SPIN_LIMIT) {
       if (abort_flag) atomicExch(abort_flag, 1);
       return false;
@@ -1734,7 +1746,7 @@ __device__ __forceinline__ void tail_sweep(const TL<V>& level, V* xs, int gg, in
     if (last) {
       if (XM == X_GLOBAL) cluster_wait();
       if (XM == X_CTA) __syncthreads();
-      if (XM == X_CLUSTER) mbar_wait(xb.bar + done, xb.parity, xb.abort);
+      if (XM == X_CLUSTER) mbar_wait<true>(xb.bar + done, xb.parity, xb.abort);
     }
   };
 #pragma unroll 1
