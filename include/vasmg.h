@@ -446,6 +446,13 @@ const char* vasmg_last_error_detail(void);
  * was satisfied, which cannot happen. */
 int vasmg_probe_wait_timeout(double* elapsed_ms);
 
+/* The tail's waits on a hierarchy of the FP32 mode in 2D: runs its tail with a
+ * cluster whose last CTA sends none of its rows.  The other CTAs' waits give up,
+ * the launch ends within a few seconds and the call returns VASMG_ERR_TIMEOUT;
+ * the hierarchy stays usable.  VASMG_ERR_UNSUPPORTED in other modes, and where
+ * the tail has one CTA or no level whose rows are sent. */
+int vasmg_probe_tail_wait(vasmg_handle h, double* elapsed_ms);
+
 #ifdef __cplusplus
 }
 #endif

@@ -665,4 +665,12 @@ int vasmg_probe_wait_timeout(double* elapsed_ms) {
   VASMG_API_END
 }
 
+int vasmg_probe_tail_wait(vasmg_handle h, double* elapsed_ms) {
+  if (!h) return VASMG_ERR_INVALID_ARG;
+  VASMG_API_BEGIN
+  join_user(h->c);
+  return probe_tail_wait(h->c, elapsed_ms);
+  VASMG_API_END
+}
+
 }  // extern "C"

@@ -262,6 +262,8 @@ struct EngineBase {
   // the engine's view for a batched launch; false unless the V-cycle has FP32
   // vectors and is the plain V-cycle
   virtual bool batch_view(EngineView<float>* v) = 0;
+  // the tail with rows that one CTA never sends: VASMG_ERR_TIMEOUT
+  virtual int probe_tail(double* ms) = 0;
   virtual int storage() const = 0;  // 0 FP64, 1 FP32, 2 BF16 operator values
 };
 
@@ -1206,6 +1208,47 @@ struct Engine : EngineBase {
   void tail(int l0, cudaStream_t s) {
     TailArgs<V> ta;
     const size_t smem = layout_tail(ta, l0);
+    launch_tail(tail_kernel<D, V, S>, ta, smem, s);
+    ++launch_counter;
+  }
+  // One cluster of FP32 2D hierarchies' tails (the kernel is built for these)
+  // whose last CTA sends nothing: the others' waits run out, they leave the
+  // sweeps, and the launch ends with the abort flag up.
+  int probe_tail(double* ms) override {
+    if constexpr (D == 2 && std::is_same<S, float>::value) {
+      cudaStream_t s = c->stream;
+      TailArgs<V> ta;
+      const size_t smem = layout_tail(ta, lt);
+      bool copies = false;
+      for (int l = ta.l0; l < ta.ls; ++l) copies |= ta.lv[l].xoff >= 0;
+      VASMG_CHECK(nct > 1 && copies, VASMG_ERR_UNSUPPORTED, "no rows are sent between the tail's CTAs");
+      VASMG_CUDA(cudaFuncSetAttribute(tail_drop_kernel<D, V, S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      TAIL_SMEM_MAX));
+      if (nct > 8)
+        VASMG_CUDA(cudaFuncSetAttribute(tail_drop_kernel<D, V, S>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+      clear_abort(s);
+      cudaEvent_t e0, e1;
+      VASMG_CUDA(cudaEventCreate(&e0));
+      VASMG_CUDA(cudaEventCreate(&e1));
+      VASMG_CUDA(cudaEventRecord(e0, s));
+      launch_tail(tail_drop_kernel<D, V, S>, ta, smem, s);
+      VASMG_CUDA(cudaEventRecord(e1, s));
+      VASMG_CUDA(cudaEventSynchronize(e1));
+      float t = 0.0f;
+      VASMG_CUDA(cudaEventElapsedTime(&t, e0, e1));
+      cudaEventDestroy(e0);
+      cudaEventDestroy(e1);
+      if (ms) *ms = t;
+      const bool gave_up = read_abort(s) != 0;
+      clear_abort(s);
+      return gave_up ? VASMG_ERR_TIMEOUT : VASMG_OK;
+    } else {
+      (void)ms;
+      return VASMG_ERR_UNSUPPORTED;
+    }
+  }
+  template <typename K>
+  void launch_tail(K kern, const TailArgs<V>& ta, size_t smem, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(nct);
     cfg.blockDim = dim3(tail_threads<D, V>());
@@ -1218,8 +1261,7 @@ struct Engine : EngineBase {
     at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    VASMG_CUDA(cudaLaunchKernelEx(&cfg, tail_kernel<D, V, S>, ta));
-    ++launch_counter;
+    VASMG_CUDA(cudaLaunchKernelEx(&cfg, kern, ta));
   }
   // V-cycle from level l0 (b_{l0} set, result in x_{l0}).
   void vcycle(int l0, cudaStream_t s) {
@@ -1980,6 +2022,10 @@ int probe_wait_timeout(double* elapsed_ms) {
   const std::vector<int32_t> f = flags.download();
   if (f[1] == 2 && f[0] == 1) return VASMG_ERR_TIMEOUT;
   return f[1] == 1 ? VASMG_OK : VASMG_ERR_CUDA;
+}
+
+int probe_tail_wait(Ctx& c, double* elapsed_ms) {
+  return c.eng ? c.eng->probe_tail(elapsed_ms) : VASMG_ERR_UNSUPPORTED;
 }
 
 void dense_level_info(Ctx& c, int* kd, int* dn) {

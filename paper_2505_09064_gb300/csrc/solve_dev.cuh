@@ -1649,6 +1649,15 @@ struct XBars {
   int* cs;          // shared memory for the level's colour starts (the row after next's address waits for them)
 };
 
+// After the last cluster barrier nothing is sent any more.  A CTA whose waits were
+// all satisfied has every row that was sent to it; one that gave up has not
+// counted them, and stays for the millisecond in which the rows still on their
+// way land (they take microseconds).
+__device__ __forceinline__ void settle_rows() {
+#pragma unroll 1
+  for (int t = 0; t < 100; ++t) __nanosleep(10000);
+}
+
 // One multicolour sweep of a tail level (MODE 0: forward from zero, MODE 1:
 // backward).  Group gg of NG handles rows base + gg.  Ahead of a colour each
 // lane has loaded its entries of the group's next two rows (an L2 round trip
@@ -1662,8 +1671,13 @@ struct XBars {
 // the barrier before its first row's gathers, behind the loads of the first
 // rows' entries.  (The forward sweep writes every entry before it is read, and a
 // cluster barrier separates it from the last reads of the copies.)
+// Returns false, for the whole CTA, if a wait of an X_CLUSTER sweep gave up: the
+// warp leaves the sweep, so rows are missing in every copy and the mbarriers'
+// phases are open.  The CTA then takes part in no further X_CLUSTER sweep
+// (another arrival on an open phase would break its count); the others' waits
+// see the abort flag.
 template <int D, int G, typename V, typename S, int MODE, int XM>
-__device__ __forceinline__ void tail_sweep(const TL<V>& level, V* xs, int gg, int NG, int lane, const XBars& xb, bool out) {
+__device__ __forceinline__ bool tail_sweep(const TL<V>& level, V* xs, int gg, int NG, int lane, const XBars& xb, bool out) {
   constexpr int NPF = tail_npf<D, V>();
   constexpr bool LC = XM == X_CTA;
   const TL<V> L = level;  // in registers: the asm statements' memory clobbers would have it loaded again at every step
@@ -1714,6 +1728,7 @@ __device__ __forceinline__ void tail_sweep(const TL<V>& level, V* xs, int gg, in
   load(nxt, range(nxt), sb);
   RowEnds sg = range(nn);
   if constexpr (XM == X_CLUSTER && MODE == 1) cluster_wait();
+  bool ok = true;
   // the row at `cur`, then the entries of the one two ahead into its registers
   auto step = [&](TailRow<D, V, S, NPF>& st) __attribute__((always_inline)) {
     const int row = cur.base + gg;
@@ -1746,15 +1761,17 @@ __device__ __forceinline__ void tail_sweep(const TL<V>& level, V* xs, int gg, in
     if (last) {
       if (XM == X_GLOBAL) cluster_wait();
       if (XM == X_CTA) __syncthreads();
-      if (XM == X_CLUSTER) mbar_wait<true>(xb.bar + done, xb.parity, xb.abort);
+      if (XM == X_CLUSTER) ok = __all_sync(0xffffffffu, mbar_wait<true>(xb.bar + done, xb.parity, xb.abort));
     }
   };
 #pragma unroll 1
-  while (cur.i < C) {
+  while (cur.i < C && ok) {
     step(sa);
-    if (cur.i >= C) break;
+    if (cur.i >= C || !ok) break;
     step(sb);
   }
+  if constexpr (XM == X_CLUSTER) ok = __syncthreads_and(ok);
+  return ok;
 }
 
 // r = -(upper part) x of a tail level, the next two rows' entries, and the range
@@ -1975,8 +1992,9 @@ __device__ __forceinline__ void dense_level_rows(const TailArgs<float>& A, float
 // that a colour of a few dozen rows spreads over all of them.  The levels below
 // are the dense level's product, or run on CTA 0 alone between two cluster
 // barriers.  Every group runs the same number of loop trips so the shuffles
-// stay converged.
-template <int D, typename V, typename S>
+// stay converged.  DROP: the last CTA sends none of its rows, as one whose waits
+// gave up (vasmg_probe_tail_wait).
+template <int D, typename V, typename S, bool DROP = false>
 __device__ __forceinline__ void tail_run(const TailArgs<V>& A) {
   extern __shared__ __align__(16) unsigned char tail_smem[];
   __shared__ __align__(8) unsigned long long xbar[TAIL_MAX_COLOURS];
@@ -2003,11 +2021,12 @@ __device__ __forceinline__ void tail_run(const TailArgs<V>& A) {
   for (int i = threadIdx.x; i < A.nbar; i += blockDim.x) mbar_init(xbar + i, 1);
   mbar_fence_init();
   cluster_sync_all();
+  bool ok = !DROP || rank + 1 < nct;  // no wait of this CTA has given up
 #pragma unroll 1
   for (int l = l0; l < ls; ++l) {
     set_level(l);
     if (L.xoff >= 0) {
-      tail_sweep<D, G, V, S, 0, X_CLUSTER>(L, sm + L.xoff, gg, NG, lane, xb, false);
+      if (ok) ok = tail_sweep<D, G, V, S, 0, X_CLUSTER>(L, sm + L.xoff, gg, NG, lane, xb, false);
       xb.parity ^= 1u;
       tail_residual<D, G, V, S, X_CLUSTER>(L, sm + L.xoff, gg, NG, lane);
     } else {
@@ -2038,7 +2057,10 @@ __device__ __forceinline__ void tail_run(const TailArgs<V>& A) {
       tail_prolong_xs<D, V>(L, sm + L.xoff, xsc, tid, NT);
       cluster_sync_all();
       tail_fetch_xs<D, V>(L, sm + L.xoff);
-      tail_sweep<D, G, V, S, 1, X_CLUSTER>(L, sm + L.xoff, gg, NG, lane, xb, l == l0 || A.lv[l - 1].xoff < 0);
+      if (ok)
+        ok = tail_sweep<D, G, V, S, 1, X_CLUSTER>(L, sm + L.xoff, gg, NG, lane, xb, l == l0 || A.lv[l - 1].xoff < 0);
+      else
+        cluster_wait();
       xb.parity ^= 1u;
     } else {
       // x of a coarser level that was swept in the CTAs' copies comes from global
@@ -2052,11 +2074,17 @@ __device__ __forceinline__ void tail_run(const TailArgs<V>& A) {
   }
   // no CTA leaves while another may still send to it
   cluster_sync_all();
+  if (!ok) settle_rows();
 }
 
 template <int D, typename V, typename S>
 __global__ void __launch_bounds__(tail_threads<D, V>(), 1) tail_kernel(const __grid_constant__ TailArgs<V> A) {
   tail_run<D, V, S>(A);
+}
+
+template <int D, typename V, typename S>
+__global__ void __launch_bounds__(tail_threads<D, V>(), 1) tail_drop_kernel(const __grid_constant__ TailArgs<V> A) {
+  tail_run<D, V, S, true>(A);
 }
 
 // The dense level's matrix, column by column: CTA j runs the one-CTA V-cycle

@@ -34,7 +34,8 @@ EXPORTED = ["vasmg_default_options", "vasmg_setup", "vasmg_assemble_load", "vasm
             "vasmg_last_launch_count", "vasmg_destroy", "vasmg_error_string", "vasmg_last_error_detail",
             "vasmg_coarse_solve_noalloc", "vasmg_server_default_opts", "vasmg_server_create",
             "vasmg_server_submit", "vasmg_server_poll", "vasmg_server_destroy", "vasmg_update_data",
-            "vasmg_probe_wait_timeout", "vasmg_probe_fp64_rate", "vasmg_solve_multi", "vasmg_time_kernel_multi"]
+            "vasmg_probe_wait_timeout", "vasmg_probe_tail_wait", "vasmg_probe_fp64_rate",
+            "vasmg_solve_multi", "vasmg_time_kernel_multi"]
 
 OK, NOT_CONVERGED, PENDING = 0, 1, 2
 NOALLOC_MAX_DOFS = 4096  # VASMG_NOALLOC_MAX_DOFS
@@ -123,6 +124,8 @@ def load():
     lib.vasmg_last_error_detail.restype = C.c_char_p
     lib.vasmg_probe_wait_timeout.argtypes = [C.POINTER(C.c_double)]
     lib.vasmg_probe_wait_timeout.restype = C.c_int
+    lib.vasmg_probe_tail_wait.argtypes = [P, C.POINTER(C.c_double)]
+    lib.vasmg_probe_tail_wait.restype = C.c_int
     lib.vasmg_probe_fp64_rate.argtypes = [C.POINTER(C.c_double), C.POINTER(C.c_double)]
     lib.vasmg_probe_fp64_rate.restype = C.c_int
     _lib = lib
@@ -261,6 +264,14 @@ def vasmg_probe_wait_timeout():
     (return code, kernel milliseconds).  The code is VASMG_ERR_TIMEOUT."""
     ms = C.c_double()
     rc = load().vasmg_probe_wait_timeout(C.byref(ms))
+    return rc, ms.value
+
+
+def vasmg_probe_tail_wait(h):
+    """Run the tail of a 2D FP32 hierarchy with rows that one CTA never sends;
+    returns (return code, kernel milliseconds).  The code is VASMG_ERR_TIMEOUT."""
+    ms = C.c_double()
+    rc = load().vasmg_probe_tail_wait(h, C.byref(ms))
     return rc, ms.value
 
 
