@@ -446,6 +446,17 @@ const char* vasmg_last_error_detail(void);
  * was satisfied, which cannot happen. */
 int vasmg_probe_wait_timeout(double* elapsed_ms);
 
+/* The same for each of the sweeps' bounded waits: a region's stage word (2D
+ * levels, and 8 right-hand sides in 3D), one or several tagged values (3D), and
+ * a chunk of the staged operator.  Each gives up after 0.1-3 s. */
+enum {
+  VASMG_WAIT_STAGE = 0,
+  VASMG_WAIT_TAGGED = 1,
+  VASMG_WAIT_TAGGED_ALL = 2,
+  VASMG_WAIT_CHUNK = 3
+};
+int vasmg_probe_wait(int32_t which, double* elapsed_ms);
+
 /* The tail's waits on a hierarchy of the FP32 mode in 2D: runs its tail with a
  * cluster whose last CTA sends none of its rows.  The other CTAs' waits give up,
  * the launch ends within a few seconds and the call returns VASMG_ERR_TIMEOUT;

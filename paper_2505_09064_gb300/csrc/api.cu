@@ -661,7 +661,14 @@ int vasmg_probe_fp64_rate(double* tflops, double* ms) {
 
 int vasmg_probe_wait_timeout(double* elapsed_ms) {
   VASMG_API_BEGIN
-  return probe_wait_timeout(elapsed_ms);
+  return probe_wait(VASMG_WAIT_STAGE, elapsed_ms);
+  VASMG_API_END
+}
+
+int vasmg_probe_wait(int32_t which, double* elapsed_ms) {
+  if (which < VASMG_WAIT_STAGE || which > VASMG_WAIT_CHUNK) return VASMG_ERR_INVALID_ARG;
+  VASMG_API_BEGIN
+  return probe_wait(which, elapsed_ms);
   VASMG_API_END
 }
 

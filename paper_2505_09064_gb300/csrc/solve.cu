@@ -1926,13 +1926,36 @@ void staged_info(Ctx& c, int level, int64_t* v) {
   if (c.eng) c.eng->staged(level, v);
 }
 
-// The bounded wait on its own: one CTA waits for a stage word that nothing
-// publishes.  The wait must give up after SPIN_LIMIT polls, raise the abort
-// flag and return; *result is 1 if the wait was satisfied, 2 if it gave up.
-__global__ void wait_probe_kernel(const int* __restrict__ list, const unsigned long long* word, int* abort_flag,
+// The bounded waits on their own: one CTA waits for a stage word that nothing
+// publishes, for words that never carry the tag, or for a chunk that nothing
+// copies (`words`: 32 bytes of zeros).  A wait must give up after its limit,
+// raise the abort flag and return; *result is 1 if it was satisfied, 2 if it
+// gave up.
+__global__ void wait_probe_kernel(int which, const int* __restrict__ list, const uint4* words, int* abort_flag,
                                   int* result) {
-  const bool ok = wait_regions(list, 1, word, 1u, 1u, abort_flag);
-  if (threadIdx.x == 0) *result = ok ? 1 : 2;
+  __shared__ __align__(8) unsigned long long bar;
+  if (threadIdx.x == 0) mbar_init(&bar, 1);
+  mbar_fence_init();
+  __syncthreads();
+  constexpr unsigned TAG = 1u;
+  bool dead = false;
+  if (which == VASMG_WAIT_STAGE) {
+    dead = !wait_regions(list, 1, reinterpret_cast<const unsigned long long*>(words), 1u, 1u, abort_flag);
+  } else if (which == VASMG_WAIT_TAGGED) {
+    unsigned u[4];
+    ld_word(words, u);
+    wait_word(words, TAG, u, abort_flag, dead);
+  } else if (which == VASMG_WAIT_TAGGED_ALL) {
+    const int v[2] = {0, 1};
+    unsigned u[2][1][4];
+    ld_word(words, u[0][0]);
+    ld_word(words + 1, u[1][0]);
+    wait_words<2, 1>(words, v, 3u, TAG, u, abort_flag, dead);
+  } else {
+    dead = !mbar_wait(&bar, 0u, abort_flag);
+  }
+  dead = __any_sync(0xffffffffu, dead);
+  if (threadIdx.x == 0) *result = dead ? 2 : 1;
 }
 
 // FP64 FMA throughput: each thread runs FMA_CHAINS independent chains of
@@ -1991,17 +2014,17 @@ int probe_fp64_rate(double* tflops, double* ms_out) {
   return VASMG_OK;
 }
 
-int probe_wait_timeout(double* elapsed_ms) {
+int probe_wait(int which, double* elapsed_ms) {
   cudaStream_t s = nullptr;
   VASMG_CUDA(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
   struct StreamGuard {
     cudaStream_t s;
     ~StreamGuard() { cudaStreamDestroy(s); }
   } guard{s};
-  DevBuf<unsigned long long> word;
+  DevBuf<uint4> words;
   DevBuf<int32_t> list, flags;
-  word.alloc(1, s);
-  word.zero();
+  words.alloc(2, s);
+  words.zero();
   list.alloc(1, s);
   list.zero();
   flags.alloc(2, s);
@@ -2010,7 +2033,7 @@ int probe_wait_timeout(double* elapsed_ms) {
   VASMG_CUDA(cudaEventCreate(&e0));
   VASMG_CUDA(cudaEventCreate(&e1));
   VASMG_CUDA(cudaEventRecord(e0, s));
-  wait_probe_kernel<<<1, 32, 0, s>>>(list.get(), word.get(), flags.get(), flags.get() + 1);
+  wait_probe_kernel<<<1, 32, 0, s>>>(which, list.get(), words.get(), flags.get(), flags.get() + 1);
   check_launch("wait_probe");
   VASMG_CUDA(cudaEventRecord(e1, s));
   VASMG_CUDA(cudaEventSynchronize(e1));

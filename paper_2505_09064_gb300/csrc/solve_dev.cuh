@@ -864,15 +864,17 @@ __device__ __forceinline__ bool mbar_test(unsigned long long* b, unsigned parity
   return done != 0;
 }
 // Wait for the phase of the given parity to complete.  Gives up (false)
-// after SPIN_LIMIT polls (after the first 64, 64 ns apart), raising the abort
+// after MBAR_LIMIT polls (after the first 64, 64 ns apart), raising the abort
 // flag, or soon after another wait raised it (read every 256 polls; never
-// when abort_flag is null).
+// when abort_flag is null).  The hardware holds a poll that fails (1.5 us, at
+// cluster scope 4 us), so a wait ends after about a second.
+constexpr int MBAR_LIMIT = SPIN_LIMIT / 4;
 template <bool CLUSTER = false>
 __device__ __forceinline__ bool mbar_wait(unsigned long long* b, unsigned parity, int* abort_flag) {
 #pragma unroll 1
   for (int spins = 0;; ++spins) {
     if (mbar_test<CLUSTER>(b, parity)) return true;
-    if (spins >= SPIN_LIMIT) {
+    if (spins >= MBAR_LIMIT) {
       if (abort_flag) atomicExch(abort_flag, 1);
       return false;
     }

@@ -26,6 +26,7 @@ PRECISIONS = {"fp64": VASMG_FP64, "fp32": VASMG_FP32_VCYCLE, "bf16": VASMG_FP32_
  EXPORT_DENSE, EXPORT_LANES, EXPORT_STAGED) = (0, 1, 3, 4, 5, 6, 7, 8, 9, 10, 11, 12, 13, 14, 15, 16, 17, 18, 19)
 OP_MATVEC, OP_SMOOTH_FWD, OP_SMOOTH_BWD, OP_RESIDUAL, OP_RESTRICT, OP_PROLONG, OP_COARSE, OP_VCYCLE, OP_PRECOND = range(9)
 KERNEL_SPMV64, KERNEL_SWEEP, KERNEL_VCYCLE, KERNEL_DOWN, KERNEL_UP = 0, 1, 2, 3, 4
+WAIT_STAGE, WAIT_TAGGED, WAIT_TAGGED_ALL, WAIT_CHUNK = range(4)
 KERNEL_FWD_SWEEP, KERNEL_RESIDUAL, KERNEL_RESTRICT, KERNEL_PROLONG, KERNEL_TAIL = 5, 6, 7, 8, 9
 
 # symbols declared in include/vasmg.h
@@ -34,7 +35,7 @@ EXPORTED = ["vasmg_default_options", "vasmg_setup", "vasmg_assemble_load", "vasm
             "vasmg_last_launch_count", "vasmg_destroy", "vasmg_error_string", "vasmg_last_error_detail",
             "vasmg_coarse_solve_noalloc", "vasmg_server_default_opts", "vasmg_server_create",
             "vasmg_server_submit", "vasmg_server_poll", "vasmg_server_destroy", "vasmg_update_data",
-            "vasmg_probe_wait_timeout", "vasmg_probe_tail_wait", "vasmg_probe_fp64_rate",
+            "vasmg_probe_wait_timeout", "vasmg_probe_wait", "vasmg_probe_tail_wait", "vasmg_probe_fp64_rate",
             "vasmg_solve_multi", "vasmg_time_kernel_multi"]
 
 OK, NOT_CONVERGED, PENDING = 0, 1, 2
@@ -124,6 +125,8 @@ def load():
     lib.vasmg_last_error_detail.restype = C.c_char_p
     lib.vasmg_probe_wait_timeout.argtypes = [C.POINTER(C.c_double)]
     lib.vasmg_probe_wait_timeout.restype = C.c_int
+    lib.vasmg_probe_wait.argtypes = [C.c_int32, C.POINTER(C.c_double)]
+    lib.vasmg_probe_wait.restype = C.c_int
     lib.vasmg_probe_tail_wait.argtypes = [P, C.POINTER(C.c_double)]
     lib.vasmg_probe_tail_wait.restype = C.c_int
     lib.vasmg_probe_fp64_rate.argtypes = [C.POINTER(C.c_double), C.POINTER(C.c_double)]
@@ -264,6 +267,13 @@ def vasmg_probe_wait_timeout():
     (return code, kernel milliseconds).  The code is VASMG_ERR_TIMEOUT."""
     ms = C.c_double()
     rc = load().vasmg_probe_wait_timeout(C.byref(ms))
+    return rc, ms.value
+
+
+def vasmg_probe_wait(which: int):
+    """vasmg_probe_wait_timeout for the wait `which` (WAIT_*)."""
+    ms = C.c_double()
+    rc = load().vasmg_probe_wait(which, C.byref(ms))
     return rc, ms.value
 
 

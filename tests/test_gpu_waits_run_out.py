@@ -1,7 +1,10 @@
-"""The bounded device waits give up, without a GPU fault.
+"""Every bounded device wait gives up, without a GPU fault.
 
-The tail's waits run out inside the tail itself, in a cluster whose last CTA
-sends none of its rows: the other CTAs leave their sweeps, take part in no
+The waits of the sweeps (a region's stage word, one tagged value, several
+tagged values at once, a chunk of the staged operator) run in one CTA against
+words that nothing writes: each must report VASMG_ERR_TIMEOUT after a bounded
+time.  The tail's waits run out inside the tail itself, in a cluster whose last
+CTA sends none of its rows: the other CTAs leave their sweeps, take part in no
 further one, and the launch ends.  Afterwards the same hierarchy gives the same
 bits as before.
 """
@@ -23,6 +26,18 @@ def built():
     __graft_entry__.build()
     torch.cuda.set_device(0)
     return True
+
+
+@pytest.mark.parametrize("which", [vasmg.WAIT_STAGE, vasmg.WAIT_TAGGED, vasmg.WAIT_TAGGED_ALL, vasmg.WAIT_CHUNK])
+def test_wait_gives_up(built, which):
+    rc, ms = vasmg.vasmg_probe_wait(which)
+    assert rc == vasmg.VASMG_ERR_TIMEOUT
+    assert 1.0 < ms < 10000.0
+
+
+def test_unknown_wait_is_refused(built):
+    assert vasmg.vasmg_probe_wait(4)[0] == vasmg.VASMG_ERR_INVALID_ARG
+    assert vasmg.vasmg_probe_wait(-1)[0] == vasmg.VASMG_ERR_INVALID_ARG
 
 
 @pytest.mark.parametrize("n", [33, 64, 220])
