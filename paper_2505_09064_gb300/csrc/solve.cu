@@ -311,7 +311,7 @@ struct Engine : EngineBase {
   std::vector<int> G;
   std::vector<DevBuf<int32_t>> cs_dev, rs_dev, nb_rp, nb;
   std::vector<DevBuf<unsigned long long>> pg_d, pg_u;
-  std::vector<DevBuf<uint4>> xt;  // 3D region levels: the staged sweeps' tagged values
+  std::vector<DevBuf<uint4>> xt;  // levels with a staged copy (3D): the staged sweeps' tagged values
   std::vector<i64> nnz_lo;        // lower-part (earlier colour) blocks per level
   std::vector<DevBuf<int32_t>> rpl_dev, rph_dev, cil_dev, cih_dev;
   std::vector<DevBuf<S>> offl_dev, offh_dev;
@@ -476,11 +476,6 @@ struct Engine : EngineBase {
     v.nb = nb[l].get();
     v.pg_d = pg_d[l].get();
     v.pg_u = pg_u[l].get();
-    if constexpr (D == 3) {
-      xt[l].alloc(std::max<i64>(1, c->S[l].nv) * xt_words<V>(), s);
-      xt[l].zero();  // no launch's tag is 0
-      v.xt = xt[l].get();
-    }
   }
 
   // New operator values on the same structure: the level-0 FP64 SELL copy
@@ -755,6 +750,11 @@ struct Engine : EngineBase {
       const int NG = STG_T / g;
       VASMG_CHECK(nv < STG_NONE, VASMG_ERR_UNSUPPORTED, "level too large for the staged sweep");
       const std::vector<int> RS = rs_dev[l].download();
+      if (!xt[l].n) {
+        xt[l].alloc(sl.nv * xt_words<V>(), s);
+        xt[l].zero();  // no launch's tag is 0
+        lv[l].xt = xt[l].get();
+      }
       for (int m = 0; m < 2; ++m) {
         Staged& st = stg[m][l];
         if (st.G == g) continue;

@@ -797,7 +797,8 @@ struct MultiEngine : MultiBase {
   using V = float;
   EngineView<V> v;
   int cap = 0;                        // right-hand sides the buffers hold (2, 4 or 8)
-  std::vector<DevBuf<uint4>> xtm;     // 3D region levels: the staged sweeps' tagged values
+  std::vector<DevBuf<uint4>> xtm;     // levels with a staged copy: the tagged values (allocate_tags)
+  int tag_cap = 0;                    // right-hand sides they hold (0, 2 or 4)
   // the tail's vectors and arguments of every right-hand side
   DevBuf<V> tvec;
   DevBuf<double> ty;
@@ -852,12 +853,6 @@ struct MultiEngine : MultiBase {
       xm[l].zero();
       bm[l].zero();
       rm[l].zero();
-      // a pass with KR takes the first nv KR words; the epochs in the tags go
-      // on from pass to pass and are shared with the single sweeps
-      if (D == 3 && v.lv[l].xt) {
-        xtm[l].alloc(std::max<i64>(1, v.nv[l]) * kr, s);
-        xtm[l].zero();
-      }
     }
     const i64 n = n0();
     U.alloc(n * kr, s);
@@ -878,6 +873,29 @@ struct MultiEngine : MultiBase {
     if (!host_sc) VASMG_CUDA(cudaMallocHost((void**)&host_sc, sizeof(Scalars) * KMAX));
     if (!host_ctl) VASMG_CUDA(cudaMallocHost((void**)&host_ctl, sizeof(int) * 2));
     cap = kr;
+  }
+
+  // The tagged values for passes of up to KR right-hand sides, if those use tags:
+  // 16 bytes per vertex and right-hand side, which passes of 8 never read.  A
+  // pass takes the first nv KR words of a level; the epochs in the tags go on
+  // from pass to pass and are shared with the single sweeps.
+  template <int KR>
+  void allocate_tags() {
+    if (D != 3 || !stgm_tags(KR) || KR <= tag_cap) return;
+    for (int t = slot(2); t <= slot(4); ++t) {  // these graphs hold the words' addresses
+      if (exec_while[t]) cudaGraphExecDestroy(exec_while[t]);
+      if (exec_body[t]) cudaGraphExecDestroy(exec_body[t]);
+      exec_while[t] = exec_body[t] = nullptr;
+    }
+    cudaStream_t s = v.stream;
+    VASMG_CUDA(cudaStreamSynchronize(s));
+    tag_cap = 0;
+    for (int l = 0; l < v.L; ++l)
+      if (v.lv[l].xt) {
+        xtm[l].alloc(v.nv[l] * KR, s);
+        xtm[l].zero();  // no launch's tag is 0
+      }
+    tag_cap = KR;
   }
 
   // level l's view with the multi vectors of KR right-hand sides
@@ -1130,6 +1148,7 @@ struct MultiEngine : MultiBase {
   template <int KR>
   void set_attributes() {
     tail_cluster<KR>();
+    allocate_tags<KR>();
     // every region of a level must be resident at once: the multi sweep CTAs
     // must fit as many per SM as the single sweeps' regions need
     int bd = 0, bu = 0;
