@@ -226,6 +226,7 @@ int vasmg_setup(const vasmg_problem* pb, const vasmg_options* opt, vasmg_handle*
   c.C.resize(1);
   setup_assemble(c);
   setup_tree(c);
+  if (c.any_wide.n) c.any_wide_host = c.any_wide.download();
   setup_colour_and_solve_levels(c);
   setup_solver_state(c);
   VASMG_CUDA(cudaStreamSynchronize(s));

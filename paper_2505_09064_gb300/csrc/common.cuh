@@ -139,6 +139,7 @@ struct CanonLevel {
   DevBuf<int32_t> rp, ci;
   DevBuf<double> v;
   DevBuf<uint8_t> dead;         // nv*d
+  DevBuf<uint8_t> wide;         // level >= 1: rows whose Galerkin sum gal_wide_kernel takes
   DevBuf<u64> lat;              // level >= 1: lattice-corner keys
   i64 ncells = 0;
   DevBuf<u64> cell_start;       // level >= 1: cells sorted by start key (d*K bits)
@@ -222,6 +223,10 @@ struct Ctx {
   DevBuf<uint8_t> leaf_depth;   // per input vertex
   DevBuf<u64> leaf_start;       // per input vertex (cell start key)
   std::vector<CanonLevel> C;
+  // whether the Galerkin product of level l has rows for gal_wide_kernel; the
+  // host's copy is there once the hierarchy is built
+  DevBuf<int32_t> any_wide;
+  std::vector<int32_t> any_wide_host;
   std::vector<SolveLevel> S;
   // coarsest dense factor (FP64), in solve order of the last level
   i64 nc = 0;

@@ -101,7 +101,9 @@ __global__ void low32_i_kernel(const u64* __restrict__ k, i64 n, int32_t* __rest
 
 // The row S of a coarse row is kept in a hash table of fine columns in shared
 // memory: slots, of which at most 3/4 may be taken.  A row that reaches more
-// columns (measured: at most 350 in 3D) is summed by gal_row_direct.
+// columns (with the default leaf thresholds, at most 470 in 3D; large thresholds
+// and vertices with many neighbours go beyond) is left to gal_wide_kernel.
+constexpr int ANY_WIDE_SLOTS = 64;  // levels with a flag of their own (a hierarchy has fewer)
 template <int D>
 constexpr int gal_slots() { return D == 2 ? 256 : 1024; }
 template <int D>
@@ -122,39 +124,80 @@ __device__ __forceinline__ unsigned gal_alive(const uint8_t* __restrict__ fdead,
   return f;
 }
 
-// Row I summed term by term, w_iI (M A_l M)_ij w_jJ, by one thread per block of
-// the row (the columns j it needs are found by scanning).
+// The coarse rows that the table could not hold (wide): a warp per block (I, J),
+// which sums w_iI (M A_l M)_ij w_jJ over R's row J.  Groups of SUB lanes take one
+// fine column j each at a time, and their lanes the fine rows i of j's pattern (7
+// in 2D and 15 in 3D on a mesh; the pattern is symmetric); w_iI is looked up in
+// P's row i, and block (i, j), where it counts, by bisection.  No two warps meet,
+// and the sum's order is fixed: a lane's terms, then the xor tree.
+// Bound by the latency of the look-ups, so as many warps as there are blocks take
+// part.  vasmg_update_data, against a thread per block of the row that walked all
+// the row's terms (and against the sum of every term into the row that preceded
+// the table): 2D 200^2 with leaf threshold 64 3.34 -> 1.32 ms (2.0), 1000 29.8 ->
+// 1.88 (13.0); 3D 33^3 with 64 30.7 -> 8.7 (26.9), 300 57.2 -> 7.9 (23.7); a disc
+// around a vertex with 1100 neighbours 21.7 -> 10.0 (12.8).
 template <int D>
-__device__ void gal_row_direct(i64 I, const int32_t* __restrict__ rrp, const int32_t* __restrict__ rent,
-                               const u64* __restrict__ rkeys, const int32_t* __restrict__ prp,
-                               const int32_t* __restrict__ pci, const double* __restrict__ pw,
-                               const int32_t* __restrict__ arp, const int32_t* __restrict__ aci,
-                               const double* __restrict__ av, const uint8_t* __restrict__ fdead,
-                               const int32_t* __restrict__ crp, const int32_t* __restrict__ cci,
-                               double* __restrict__ cv) {
-  constexpr int DD = D * D;
-  for (int32_t e = crp[I] + threadIdx.x; e < crp[I + 1]; e += blockDim.x) {
-    const int32_t J = cci[e];
-    double acc[DD];
+__global__ void __launch_bounds__(256, 4) gal_wide_kernel(
+    i64 nc, const uint8_t* __restrict__ wide, const int32_t* __restrict__ any_wide, const int32_t* __restrict__ rrp,
+    const int32_t* __restrict__ rent, const u64* __restrict__ rkeys, const int32_t* __restrict__ prp,
+    const int32_t* __restrict__ pci, const double* __restrict__ pw, const int32_t* __restrict__ arp,
+    const int32_t* __restrict__ aci, const double* __restrict__ av, const uint8_t* __restrict__ fdead,
+    const int32_t* __restrict__ crp, const int32_t* __restrict__ cci, const uint8_t* __restrict__ cdead,
+    double* __restrict__ cv) {
+  constexpr int DD = D * D, SUB = D == 2 ? 8 : 16, NG = 32 / SUB;
+  __shared__ unsigned found[8];
+  if (*any_wide == 0) return;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane / SUB, sub = lane % SUB;
+  // the rows blockIdx.x, blockIdx.x + gridDim.x, ...: 256 rows' marks at once
+  for (i64 base = 0; blockIdx.x + base * gridDim.x < nc; base += 256) {
+    const i64 r = blockIdx.x + (base + threadIdx.x) * gridDim.x;
+    const unsigned m = __ballot_sync(0xffffffffu, r < nc && wide[r] != 0);
+    __syncthreads();
+    if (lane == 0) found[warp] = m;
+    __syncthreads();
+    for (int w = 0; w < 8; ++w)
+      for (unsigned left = found[w]; left; left &= left - 1) {
+        const i64 I = blockIdx.x + (base + w * 32 + __ffs(left) - 1) * gridDim.x;
+        for (int32_t e = crp[I] + warp + 8 * blockIdx.y; e < crp[I + 1]; e += 8 * gridDim.y) {
+          const int32_t J = cci[e], t1 = rrp[J + 1];
+          double acc[DD];
 #pragma unroll
-    for (int q = 0; q < DD; ++q) acc[q] = 0.0;
-    for (int32_t t = rrp[I]; t < rrp[I + 1]; ++t) {
-      const i64 i = (i64)(rkeys[t] & 0xffffffffull);
-      const double wI = pw[rent[t]];
-      const unsigned fi = gal_alive<D>(fdead, i);
-      for (int32_t k = arp[i]; k < arp[i + 1]; ++k) {
-        const i64 j = aci[k];
-        for (int32_t b = prp[j]; b < prp[j + 1]; ++b) {
-          if (pci[b] != J) continue;
-          const unsigned fj = gal_alive<D>(fdead, j);
+          for (int q = 0; q < DD; ++q) acc[q] = 0.0;
+          for (int32_t t = rrp[J] + g; t < t1; t += NG) {
+            const int32_t j = (int32_t)(rkeys[t] & 0xffffffffull);
+            const double wJ = pw[rent[t]];
+            const unsigned fj = gal_alive<D>(fdead, j);
+            const int32_t k1 = arp[j + 1];
+            for (int32_t k = arp[j] + sub; k < k1; k += SUB) {
+              const i64 i = aci[k];
+              int32_t b = prp[i];
+              const int32_t b1 = prp[i + 1];
+              while (b < b1 && pci[b] != (int32_t)I) ++b;
+              if (b == b1) continue;
+              const double wI = pw[b];
+              const unsigned fi = gal_alive<D>(fdead, i);
+              const int32_t end = arp[i + 1];
+              int32_t lo = arp[i], hi = end;
+              while (lo < hi) {
+                const int32_t mid = (lo + hi) >> 1;
+                if (aci[mid] < j) lo = mid + 1; else hi = mid;
+              }
+              if (lo == end || aci[lo] != j) continue;
 #pragma unroll
-          for (int q = 0; q < DD; ++q)
-            if (((fi >> (q / D)) & 1u) && ((fj >> (q % D)) & 1u)) acc[q] = fma(wI * av[(i64)k * DD + q], pw[b], acc[q]);
+              for (int q = 0; q < DD; ++q)
+                if (((fi >> (q / D)) & 1u) && ((fj >> (q % D)) & 1u)) acc[q] = fma(wI * av[(i64)lo * DD + q], wJ, acc[q]);
+            }
+          }
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int q = 0; q < DD; ++q) acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], o);
+          if (lane == 0)
+#pragma unroll
+            for (int q = 0; q < DD; ++q)
+              cv[(i64)e * DD + q] = J == (int32_t)I && q % (D + 1) == 0 && cdead[I * D + q / D] ? 1.0 : acc[q];
         }
       }
-    }
-#pragma unroll
-    for (int q = 0; q < DD; ++q) cv[(i64)e * DD + q] = acc[q];
   }
 }
 
@@ -171,7 +214,7 @@ __global__ void __launch_bounds__(gal_threads<D>()) gal_values_kernel(
     const int32_t* __restrict__ prp, const int32_t* __restrict__ pci, const double* __restrict__ pw,
     const int32_t* __restrict__ arp, const int32_t* __restrict__ aci, const double* __restrict__ av,
     const uint8_t* __restrict__ fdead, const int32_t* __restrict__ crp, const int32_t* __restrict__ cci,
-    double* __restrict__ cv, uint8_t* __restrict__ cdead) {
+    double* __restrict__ cv, uint8_t* __restrict__ cdead, uint8_t* __restrict__ wide, int32_t* __restrict__ any_wide) {
   constexpr int DD = D * D, SLOTS = gal_slots<D>(), T = gal_threads<D>(), EMPTY = -1;
   extern __shared__ __align__(16) unsigned char gal_mem[];
   double* S = reinterpret_cast<double*>(gal_mem);                       // [SLOTS][DD]
@@ -202,6 +245,10 @@ __global__ void __launch_bounds__(gal_threads<D>()) gal_values_kernel(
       const double wI = wn;
       const int32_t k0 = kn0, k1 = kn1;
       fetch_row(t + 1);
+      if (k1 - k0 > SLOTS - SLOTS / 4) {  // one fine row with more columns than the table takes
+        full = true;
+        break;
+      }
       const unsigned fi = gal_alive<D>(fdead, i);
       alive |= fi;
       bool over = false;
@@ -230,8 +277,10 @@ __global__ void __launch_bounds__(gal_threads<D>()) gal_values_kernel(
       full = __syncthreads_or(over);
     }
     if (full) {
-      for (int32_t t = t0; t < t1; ++t) alive |= gal_alive<D>(fdead, (i64)(rkeys[t] & 0xffffffffull));
-      gal_row_direct<D>(I, rrp, rent, rkeys, prp, pci, pw, arp, aci, av, fdead, crp, cci, cv);
+      unsigned mine = 0;
+      for (int32_t t = t0 + tid; t < t1; t += T) mine |= gal_alive<D>(fdead, (i64)(rkeys[t] & 0xffffffffull));
+#pragma unroll
+      for (int r = 0; r < D; ++r) alive |= __syncthreads_or((mine >> r) & 1u) ? 1u << r : 0u;
     } else {
       for (int32_t e = c0 + tid; e < c1; e += T) {
         const int32_t J = cci[e];
@@ -267,6 +316,10 @@ __global__ void __launch_bounds__(gal_threads<D>()) gal_values_kernel(
       }
     }
     __syncthreads();
+    if (tid == D) {
+      wide[I] = full ? 1 : 0;
+      if (full) *any_wide = 1;
+    }
     // dead coarse dofs -> identity rows (their masked column of P is empty)
     if (tid < D) {
       int32_t lo = c0, hi = c1;
@@ -334,15 +387,30 @@ void galerkin_values(Ctx& c, int l) {
   CanonLevel& g = c.C[l + 1];
   if (g.v.n != g.nnzb * d * d) g.v.alloc(g.nnzb * d * d, s);
   if (g.dead.n != g.nv * d) g.dead.alloc(g.nv * d, s);
-  auto launch = [&](auto kern, int threads, int smem) {
+  if (g.wide.n != g.nv) g.wide.alloc(g.nv, s);
+  if (!c.any_wide.n) {
+    c.any_wide.alloc(ANY_WIDE_SLOTS, s);
+    c.any_wide.zero();
+  }
+  const int slot = std::min(l, ANY_WIDE_SLOTS - 1);
+  int32_t* any = c.any_wide.get() + slot;
+  auto launch = [&](auto kern, auto wide, int threads, int smem) {
     VASMG_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     kern<<<grid_for(g.nv, 1), threads, smem, s>>>(g.nv, f.r_rp.get(), f.r_ent.get(), f.r_keys.get(), f.prp.get(),
                                                   f.pci.get(), f.pw.get(), f.rp.get(), f.ci.get(), f.v.get(),
-                                                  f.dead.get(), g.rp.get(), g.ci.get(), g.v.get(), g.dead.get());
+                                                  f.dead.get(), g.rp.get(), g.ci.get(), g.v.get(), g.dead.get(),
+                                                  g.wide.get(), any);
+    check_launch("gal_values");
+    // which levels have such rows is known once the setup is through (they follow
+    // from the structure)
+    if (!c.any_wide_host.empty() && c.any_wide_host[slot] == 0) return;
+    wide<<<dim3(grid_for(g.nv, 1, 512), 8), 256, 0, s>>>(
+        g.nv, g.wide.get(), any, f.r_rp.get(), f.r_ent.get(), f.r_keys.get(), f.prp.get(), f.pci.get(), f.pw.get(),
+        f.rp.get(), f.ci.get(), f.v.get(), f.dead.get(), g.rp.get(), g.ci.get(), g.dead.get(), g.v.get());
+    check_launch("gal_wide");
   };
-  if (d == 2) launch(gal_values_kernel<2>, gal_threads<2>(), gal_smem<2>());
-  else launch(gal_values_kernel<3>, gal_threads<3>(), gal_smem<3>());
-  check_launch("gal_values");
+  if (d == 2) launch(gal_values_kernel<2>, gal_wide_kernel<2>, gal_threads<2>(), gal_smem<2>());
+  else launch(gal_values_kernel<3>, gal_wide_kernel<3>, gal_threads<3>(), gal_smem<3>());
 }
 
 }  // namespace vasmg
