@@ -920,7 +920,7 @@ struct Engine : EngineBase {
   // For every region level, time the forward sweep, the residual and the
   // backward sweep with each G of {4, 8, 16, 32} whose kernels can hold the
   // level's region grid (CUDA events, one warm-up and three timed runs) and
-  // keep the fastest.  A level signature measured before in this process
+  // keep the fastest whose staged copy is not mostly padding.  A level signature measured before in this process
   // (by this or another handle) reuses that choice.
   void autotune_lanes() {
     cudaStream_t s = c->stream;
@@ -960,9 +960,15 @@ struct Engine : EngineBase {
         VASMG_CUDA(cudaEventSynchronize(e1));
         float ms = 0.0f;
         VASMG_CUDA(cudaEventElapsedTime(&ms, e0, e1));
-        // a staged copy of more than twice the level's blocks only where every
-        // choice needs one
-        const bool wide = stg[1].size() > (size_t)l && stg[1][l].G == g && stg[1][l].nslots > 2 * (i64)sl.nnz;
+        // A backward staged copy of more than 9/4 of the level's blocks only where
+        // every choice needs one.  On small fine levels (14 blocks a row) 16 lanes
+        // are the fastest with FP32 vectors, by 10 to 20 us a V-cycle, but their
+        // copies are mostly padding: 29^3 60 against 81 us with 4 lanes and 5.2
+        // against 1.8 slots per block, 33^3 68 / 84 us and 4.7 / 1.6, 41^3 83 / 95
+        // and 2.9 / 1.4.  The line lies above the coarser levels' fastest choice
+        // (56^3 graded level 1: 32 lanes 398 us with 2.06 slots per block, 16 lanes
+        // 477 with 1.87; the solve 3.9 % slower with 16).
+        const bool wide = stg[1].size() > (size_t)l && stg[1][l].G == g && 4 * stg[1][l].nslots > 9 * (i64)sl.nnz;
         if (best_ms == 0.0f || (wide == best_wide ? ms < best_ms : best_wide)) {
           best_ms = ms;
           best_g = g;
