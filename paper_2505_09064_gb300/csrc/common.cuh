@@ -355,7 +355,7 @@ __host__ __device__ inline long long block_index(int q, long long k, long long n
 // passes.  Used by the coarsest-level solves of the V-cycle and of
 // vasmg_coarse_solve_noalloc.
 // Up to 32 unknowns (every level coarsened to the root: 8 or 24) stay in the
-// lanes' registers, the factor's entries in flight eight steps ahead, and each
+// lanes' registers, the factor's entries loaded for eight steps at a time, and each
 // division is a product with the reciprocal (taken once, all pivots at the same
 // time) corrected by its residual: a step is four dependent FP64 operations
 // and a shuffle instead of a division and a round trip through memory.

@@ -160,12 +160,12 @@ __global__ void __launch_bounds__(256) full_residual_kernel(const __grid_constan
   for (int base = blockIdx.x * NG; base < L.nv; base += gridDim.x * NG) {
     const int row = base + g;
     const bool valid = row < L.nv;
-    RowSeg sg{0, 0, 0, 0};
+    RowSeg sg{0, 0};
     if (valid) sg = seg_range<1>(L, row);
     V acc[D];
 #pragma unroll
     for (int a = 0; a < D; ++a) acc[a] = V(0);
-    row_entries<D, G, V, S, 1, false, true>(L, sg, lane, acc);
+    row_entries<D, G, V, S, 1, true>(L, sg, lane, acc);
 #pragma unroll
     for (int o = G / 2; o > 0; o >>= 1)
 #pragma unroll

@@ -132,11 +132,14 @@ __device__ __forceinline__ void stx(V* p, V v) {
   else __stcg(p, v);
 }
 // A vector value written inside the launch by other CTAs: from L2 (.cg), or
-// (L1) through the SM's L1 cache.  L1 is used only by the region launches,
-// whose every colour step starts after a GPU-scope acquire (the neighbour
-// wait), which invalidates the SM's L1: a cached value is then never older
-// than the last step's, and within a step no value a row reads is written
-// (rows of one colour are not neighbours).  Rows of a region share most of
+// (L1) through the SM's L1 cache.  L1 is used by the region levels' launches.
+// In a sweep with stage waits every colour step starts after a GPU-scope acquire
+// (the neighbour wait), which invalidates the SM's L1: a cached value is then
+// never older than the last step's, and within a step no value a row reads is
+// written (rows of one colour are not neighbours).  A staged sweep that waits for
+// tagged values reads only old values through L1, which no row overwrites before
+// all their readers are done (see "values with tags").  Residuals and transfers
+// read what nothing writes during the launch.  Rows of a region share most of
 // their neighbours, so their gathers mostly hit L1.
 template <bool L1, typename T>
 __device__ __forceinline__ T ld_shared_vec(const T* p) {
@@ -252,65 +255,43 @@ __device__ __forceinline__ float pick(const float (&a)[D], int i) {
   return D == 2 ? (i == 0 ? a[0] : a[1]) : (i == 0 ? a[0] : (i == 1 ? a[1] : a[D - 1]));
 }
 
-// Entries of one row as a contiguous segment A[a0 .. a0 + len) of the arrays
-// the level and mode select (b0 / B are kept for a second segment and unused).
+// A row's entries [a0, a0 + len) in the arrays that the level and mode select.
 struct RowSeg {
-  int a0, la, b0, len;
+  int a0, len;
+};
+template <typename S>
+struct SegArrays {
+  const int* ci;
+  const S* off;
+  long long n;
 };
 
 // A level with split parts (LV): MODE 0 reads the lower part, MODE 2 the
-// upper part, MODE 1 (whole rows) the combined arrays; one segment each.
+// upper part, MODE 1 (whole rows) the combined arrays.
 template <int MODE, typename S, typename V>
-__device__ __forceinline__ void seg_ptrs(const LV<V>& L, const int*& ciA, const S*& offA, long long& nA,
-                                         const int*& ciB, const S*& offB, long long& nB) {
-  if (MODE == 2) {
-    ciA = L.cih;
-    offA = (const S*)L.offh;
-    nA = L.nhi;
-  } else if (MODE == 0) {
-    ciA = L.cil;
-    offA = (const S*)L.offl;
-    nA = L.nlo;
-  } else {
-    ciA = L.ci;
-    offA = (const S*)L.off;
-    nA = L.nnz;
-  }
-  ciB = ciA;
-  offB = offA;
-  nB = nA;
+__device__ __forceinline__ SegArrays<S> seg_arrays(const LV<V>& L) {
+  if (MODE == 2) return SegArrays<S>{L.cih, (const S*)L.offh, L.nhi};
+  if (MODE == 0) return SegArrays<S>{L.cil, (const S*)L.offl, L.nlo};
+  return SegArrays<S>{L.ci, (const S*)L.off, L.nnz};
 }
 template <int MODE, typename V>
 __device__ __forceinline__ RowSeg seg_range(const LV<V>& L, int row) {
   const int* p = MODE == 2 ? L.rph : (MODE == 0 ? L.rpl : L.rp);
-  RowSeg r;
-  r.a0 = __ldg(p + row);
-  r.la = __ldg(p + row + 1) - r.a0;
-  r.b0 = 0;
-  r.len = r.la;
-  return r;
+  const int a0 = __ldg(p + row);
+  return RowSeg{a0, __ldg(p + row + 1) - a0};
 }
 
 // Column index and d x d block of entry e of a row.
 template <int D, typename V, typename S>
-__device__ __forceinline__ int seg_entry(const RowSeg& r, int e, const int* ciA, const S* offA, long long nA,
-                                         const int* ciB, const S* offB, long long nB, V (&a)[D * D]) {
-  // every caller passes a single segment (la == len): B is never read
+__device__ __forceinline__ int seg_entry(const RowSeg& r, int e, const SegArrays<S>& A, V (&a)[D * D]) {
   const int k = r.a0 + e;
-  const int* cp = ciA;
-  const S* op = offA;
-  const long long n = nA;
-  (void)ciB;
-  (void)offB;
-  (void)nB;
   if constexpr (D == 2) {
-    (void)n;
-    ldv4<V, S>(op + (long long)k * 4, a);  // 2D blocks are stored contiguously
+    ldv4<V, S>(A.off + (long long)k * 4, a);  // 2D blocks are stored contiguously
   } else {
-    ldv8<V, S>(op + (long long)k * 8, a);  // components 0..7 contiguous (block_index)
-    a[8] = ldv<V, S>(op + 8 * n + k);
+    ldv8<V, S>(A.off + (long long)k * 8, a);  // components 0..7 contiguous (block_index)
+    a[8] = ldv<V, S>(A.off + 8 * A.n + k);
   }
-  return __ldg(cp + k);
+  return __ldg(A.ci + k);
 }
 
 // Gathers of a region level go through L1 (see ld_shared_vec); the cluster
@@ -329,20 +310,14 @@ constexpr bool gather_l1() { return !LC && !is_tail_level<L_t>::value; }
 // and a single (see ldx_vertex).  (Loading several entries before their
 // gathers was measured: no faster for the sweeps, which wait at their
 // barriers, and twice as slow for the residual, whose occupancy it halved.)
-template <int D, int G, typename V, typename S, int MODE, bool LC, bool PAIR3, typename L_t>
-__device__ __forceinline__ void row_entries(const L_t& L, const RowSeg& sg, int e0, V (&acc)[D]) {
-  const int* ciA;
-  const S* offA;
-  long long nA;
-  const int* ciB;
-  const S* offB;
-  long long nB;
-  seg_ptrs<MODE, S>(L, ciA, offA, nA, ciB, offB, nB);
+template <int D, int G, typename V, typename S, int MODE, bool PAIR3>
+__device__ __forceinline__ void row_entries(const LV<V>& L, const RowSeg& sg, int e0, V (&acc)[D]) {
+  const SegArrays<S> A = seg_arrays<MODE, S>(L);
   for (int e = e0; e < sg.len; e += G) {
     V blk[D * D];
-    const int j = seg_entry<D, V, S>(sg, e, ciA, offA, nA, ciB, offB, nB, blk);
+    const int j = seg_entry<D, V, S>(sg, e, A, blk);
     V xj[D];
-    ldx_vertex<D, LC, PAIR3, gather_l1<L_t, LC>()>((const V*)L.x + (long long)j * D, xj);
+    ldx_vertex<D, false, PAIR3, true>((const V*)L.x + (long long)j * D, xj);
 #pragma unroll
     for (int a = 0; a < D; ++a)
 #pragma unroll
@@ -363,35 +338,30 @@ struct RowPF {
 // Row pass split in two.  row_prefetch loads everything that nothing writes
 // during the sweep (row range, the first NPF entries of this lane, the
 // diagonal inverse and b); row_finish, called once the rows this row depends
-// on are done, gathers x and completes the row as row_pass does.
-template <int D, int G, typename V, typename S, int MODE, typename L_t, bool LC = false, int NPF>
-__device__ __forceinline__ void row_prefetch(const L_t& L, int row, bool valid, int lane, RowPF<D, V, NPF>& st) {
-  st.sg = RowSeg{0, 0, 0, 0};
+// on are done, gathers x and writes the row: x_i = D^-1 (b_i - sum), or, MODE 2,
+// r_i = -sum.
+template <int D, int G, typename V, typename S, int MODE, int NPF>
+__device__ __forceinline__ void row_prefetch(const LV<V>& L, int row, bool valid, int lane, RowPF<D, V, NPF>& st) {
+  st.sg = RowSeg{0, 0};
   if (valid) st.sg = seg_range<MODE>(L, row);
-  const int* ciA;
-  const S* offA;
-  long long nA;
-  const int* ciB;
-  const S* offB;
-  long long nB;
-  seg_ptrs<MODE, S>(L, ciA, offA, nA, ciB, offB, nB);
+  const SegArrays<S> A = seg_arrays<MODE, S>(L);
 #pragma unroll
   for (int p = 0; p < NPF; ++p) {
     const int e = lane + p * G;
     st.cj[p] = -1;
-    if (e < st.sg.len) st.cj[p] = seg_entry<D, V, S>(st.sg, e, ciA, offA, nA, ciB, offB, nB, st.a[p]);
+    if (e < st.sg.len) st.cj[p] = seg_entry<D, V, S>(st.sg, e, A, st.a[p]);
   }
   if (MODE != 2 && valid && lane < D) {
 #pragma unroll
     for (int bb = 0; bb < D; ++bb) {
       st.di[bb] = __ldg((const V*)L.dinv + (long long)(lane * D + bb) * L.nv + row);
-      st.bv[bb] = ldx<LC>((const V*)L.b + (long long)row * D + bb);
+      st.bv[bb] = ldx((const V*)L.b + (long long)row * D + bb);
     }
   }
 }
 
-template <int D, int G, typename V, typename S, int MODE, typename L_t, bool LC = false, int NPF>
-__device__ __forceinline__ void row_finish(const L_t& L, int row, bool valid, int lane, const RowPF<D, V, NPF>& st) {
+template <int D, int G, typename V, typename S, int MODE, int NPF>
+__device__ __forceinline__ void row_finish(const LV<V>& L, int row, bool valid, int lane, const RowPF<D, V, NPF>& st) {
   V acc[D];
 #pragma unroll
   for (int a = 0; a < D; ++a) acc[a] = V(0);
@@ -399,26 +369,26 @@ __device__ __forceinline__ void row_finish(const L_t& L, int row, bool valid, in
   for (int p = 0; p < NPF; ++p) {
     if (st.cj[p] >= 0) {
       V xj[D];
-      ldx_vertex<D, LC, false, gather_l1<L_t, LC>()>((const V*)L.x + (long long)st.cj[p] * D, xj);
+      ldx_vertex<D, false, false, true>((const V*)L.x + (long long)st.cj[p] * D, xj);
 #pragma unroll
       for (int a = 0; a < D; ++a)
 #pragma unroll
         for (int bb = 0; bb < D; ++bb) acc[a] += st.a[p][a * D + bb] * xj[bb];
     }
   }
-  row_entries<D, G, V, S, MODE, LC, false>(L, st.sg, lane + NPF * G, acc);
+  row_entries<D, G, V, S, MODE, false>(L, st.sg, lane + NPF * G, acc);
 #pragma unroll
   for (int o = G / 2; o > 0; o >>= 1)
 #pragma unroll
     for (int a = 0; a < D; ++a) acc[a] += __shfl_xor_sync(0xffffffffu, acc[a], o, G);
   if (!valid || lane >= D) return;
   if (MODE == 2) {
-    stx<LC>(L.r + (long long)row * D + lane, -pick<D>(acc, lane));
+    stx(L.r + (long long)row * D + lane, -pick<D>(acc, lane));
   } else {
     V s = V(0);
 #pragma unroll
     for (int bb = 0; bb < D; ++bb) s += st.di[bb] * (st.bv[bb] - acc[bb]);
-    stx<LC>(L.x + (long long)row * D + lane, s);
+    stx(L.x + (long long)row * D + lane, s);
   }
 }
 
@@ -698,30 +668,24 @@ __global__ void __launch_bounds__(df_threads<D, V>(), df_min_blocks<D, V>())
 
 // r = -(upper part) x after the zero-start forward sweep: a plain SpMV of
 // the later-colour blocks, G lanes per row, grid-strided over the rows.
-// The residual of one row of a region level (row_pass, MODE 2) with each lane's
+// The residual of one row of a region level with each lane's
 // entries taken two at a time: both blocks and both gathers in flight before
 // the products, which are added in entry order.  The kernel keeps 32 registers
 // with FP32 vectors (8 CTAs per SM): 128^3 graded, level-1 residual
 // 312 -> 291 us.
 template <int D, int G, typename V, typename S>
 __device__ __forceinline__ void residual_row_u2(const LV<V>& L, int row, bool valid, int lane) {
-  RowSeg sg{0, 0, 0, 0};
+  RowSeg sg{0, 0};
   if (valid) sg = seg_range<2>(L, row);
   V acc[D];
 #pragma unroll
   for (int a = 0; a < D; ++a) acc[a] = V(0);
-  const int* ciA;
-  const S* offA;
-  long long nA;
-  const int* ciB;
-  const S* offB;
-  long long nB;
-  seg_ptrs<2, S>(L, ciA, offA, nA, ciB, offB, nB);
+  const SegArrays<S> A = seg_arrays<2, S>(L);
   int e = lane;
   for (; e + G < sg.len; e += 2 * G) {
     V b0[D * D], b1[D * D];
-    const int j0 = seg_entry<D, V, S>(sg, e, ciA, offA, nA, ciB, offB, nB, b0);
-    const int j1 = seg_entry<D, V, S>(sg, e + G, ciA, offA, nA, ciB, offB, nB, b1);
+    const int j0 = seg_entry<D, V, S>(sg, e, A, b0);
+    const int j1 = seg_entry<D, V, S>(sg, e + G, A, b1);
     V x0[D], x1[D];
     ldx_vertex<D, false, true, true>((const V*)L.x + (long long)j0 * D, x0);
     ldx_vertex<D, false, true, true>((const V*)L.x + (long long)j1 * D, x1);
@@ -736,7 +700,7 @@ __device__ __forceinline__ void residual_row_u2(const LV<V>& L, int row, bool va
   }
   if (e < sg.len) {
     V b0[D * D];
-    const int j0 = seg_entry<D, V, S>(sg, e, ciA, offA, nA, ciB, offB, nB, b0);
+    const int j0 = seg_entry<D, V, S>(sg, e, A, b0);
     V x0[D];
     ldx_vertex<D, false, true, true>((const V*)L.x + (long long)j0 * D, x0);
 #pragma unroll
@@ -1347,7 +1311,7 @@ __global__ void coarse_kernel(CoarseArgs A, const V* b, V* x) {
   if (threadIdx.x < 32) coarse_solve_warp<V>(A, b, x);
 }
 
-// A level as the tail kernel sees it (the fields row_pass and the transfers use).
+// A level as the tail kernel sees it (the fields its rows and the transfers use).
 template <typename V>
 struct TL {
   int nv;
@@ -1375,32 +1339,15 @@ struct TL {
   V* xg;     // the same copy in global memory, written by the prolongation
 };
 
-// A tail level keeps the combined CSR: one segment, [rp, sp) lower, [sp,
-// rp+1) upper.
-template <int MODE, typename S, typename V>
-__device__ __forceinline__ void seg_ptrs(const TL<V>& L, const int*& ciA, const S*& offA, long long& nA,
-                                         const int*& ciB, const S*& offB, long long& nB) {
-  ciA = ciB = L.ci;
-  offA = offB = (const S*)L.off;
-  nA = nB = L.nnz;
-}
-// The same as its two ends (a difference taken at once would wait for the loads)
+// A tail level keeps the combined CSR, a row [rp, sp) lower, [sp, rp+1) upper:
+// the two ends of the part that MODE reads (a difference taken at once would wait
+// for the loads).
 struct RowEnds {
   int a0, a1;
 };
 template <int MODE, typename V>
 __device__ __forceinline__ RowEnds row_ends(const TL<V>& L, int row) {
   return RowEnds{MODE == 2 ? __ldg(L.sp + row) : __ldg(L.rp + row), MODE == 0 ? __ldg(L.sp + row) : __ldg(L.rp + row + 1)};
-}
-template <int MODE, typename V>
-__device__ __forceinline__ RowSeg seg_range(const TL<V>& L, int row) {
-  RowSeg r;
-  r.a0 = MODE == 2 ? __ldg(L.sp + row) : __ldg(L.rp + row);
-  const int a1 = MODE == 0 ? __ldg(L.sp + row) : __ldg(L.rp + row + 1);
-  r.la = a1 - r.a0;
-  r.b0 = 0;
-  r.len = r.la;
-  return r;
 }
 
 template <typename V>
@@ -1595,7 +1542,7 @@ __device__ __forceinline__ void tail_row_load(const TL<V>& L, int row, bool vali
 }
 
 // The row's gathers of x, all in flight together, and its sum in the order of
-// row_pass.  Returns component own_comp(lane) of x (MODE 0, 1) or r (MODE 2).
+// row_finish.  Returns component own_comp(lane) of x (MODE 0, 1) or r (MODE 2).
 template <int D, int G, typename V, typename S, int MODE, int XM, int NPF>
 __device__ __forceinline__ V tail_row_value(const TL<V>& L, const V* xs, int lane, const TailRow<D, V, S, NPF>& st) {
   constexpr bool LC = XM == X_CTA;

@@ -29,10 +29,9 @@ constexpr int DFM_THREADS = 256;    // threads of the batched sweep CTAs and of 
 constexpr int KMAX = 8;             // right-hand sides per pass
 constexpr int KG_SPMV = 4;          // right-hand sides per SpMV launch
 
-// N consecutive vector values (a vertex's KR x D entries), through L1 on the
-// region levels and from L2 on the tail's levels (see ld_shared_vec): 16-byte
-// loads when N is a multiple of 4 (the block starts on a 16-byte boundary),
-// else 8-byte loads.
+// N consecutive vector values (a vertex's KR x D entries), through L1 or from L2
+// (see ld_shared_vec): 16-byte loads when N is a multiple of 4 (the block starts
+// on a 16-byte boundary), else 8-byte loads.
 template <int N, bool L1>
 __device__ __forceinline__ void ld_vec_n(const float* p, float (&v)[N]) {
   if constexpr (N % 4 == 0) {
@@ -66,19 +65,13 @@ struct RowPFM {
 // Loads what nothing writes during the sweep: the row range, this lane's
 // first entry and the diagonal inverse row (b of the right-hand sides is
 // loaded when the row is finished, which keeps the prefetched state small).
-template <int D, int KR, typename V, typename S, int MODE, typename L_t>
-__device__ __forceinline__ void rowm_prefetch(const L_t& L, int row, bool valid, int lane, RowPFM<D, KR, V>& st) {
-  st.sg = RowSeg{0, 0, 0, 0};
+template <int D, int KR, typename V, typename S, int MODE>
+__device__ __forceinline__ void rowm_prefetch(const LV<V>& L, int row, bool valid, int lane, RowPFM<D, KR, V>& st) {
+  st.sg = RowSeg{0, 0};
   if (valid) st.sg = seg_range<MODE>(L, row);
-  const int* ciA;
-  const S* offA;
-  long long nA;
-  const int* ciB;
-  const S* offB;
-  long long nB;
-  seg_ptrs<MODE, S>(L, ciA, offA, nA, ciB, offB, nB);
+  const SegArrays<S> A = seg_arrays<MODE, S>(L);
   st.cj = -1;
-  if (lane < st.sg.len) st.cj = seg_entry<D, V, S>(st.sg, lane, ciA, offA, nA, ciB, offB, nB, st.a);
+  if (lane < st.sg.len) st.cj = seg_entry<D, V, S>(st.sg, lane, A, st.a);
   if (MODE != 2 && valid && lane < D) {
 #pragma unroll
     for (int bb = 0; bb < D; ++bb) st.di[bb] = __ldg((const V*)L.dinv + (long long)(lane * D + bb) * L.nv + row);
@@ -88,8 +81,8 @@ __device__ __forceinline__ void rowm_prefetch(const L_t& L, int row, bool valid,
 // The row's products for every right-hand side, G lanes over its entries in
 // the order e = lane, lane + G, ... (as the single sweep), the lanes' sums
 // combined by the same shuffle tree; lanes a < D then write component a.
-template <int D, int KR, typename V, typename S, int MODE, typename L_t>
-__device__ __forceinline__ void rowm_finish(const L_t& L, int row, bool valid, int lane, int G,
+template <int D, int KR, typename V, typename S, int MODE>
+__device__ __forceinline__ void rowm_finish(const LV<V>& L, int row, bool valid, int lane, int G,
                                             const RowPFM<D, KR, V>& st) {
   V acc[KR][D];
 #pragma unroll
@@ -101,7 +94,7 @@ __device__ __forceinline__ void rowm_finish(const L_t& L, int row, bool valid, i
   if (MODE != 2 && valid && lane < D) ld_vec_n<KR * D, false>((const V*)L.b + (long long)row * KR * D, bv);
   if (st.cj >= 0) {
     V xj[KR * D];
-    ld_vec_n<KR * D, gather_l1<L_t, false>()>((const V*)L.x + (long long)st.cj * KR * D, xj);
+    ld_vec_n<KR * D, true>((const V*)L.x + (long long)st.cj * KR * D, xj);
 #pragma unroll
     for (int i = 0; i < KR; ++i)
 #pragma unroll
@@ -109,18 +102,12 @@ __device__ __forceinline__ void rowm_finish(const L_t& L, int row, bool valid, i
 #pragma unroll
         for (int bb = 0; bb < D; ++bb) acc[i][a] += st.a[a * D + bb] * xj[i * D + bb];
   }
-  const int* ciA;
-  const S* offA;
-  long long nA;
-  const int* ciB;
-  const S* offB;
-  long long nB;
-  seg_ptrs<MODE, S>(L, ciA, offA, nA, ciB, offB, nB);
+  const SegArrays<S> A = seg_arrays<MODE, S>(L);
   for (int e = lane + G; e < st.sg.len; e += G) {
     V blk[D * D];
-    const int j = seg_entry<D, V, S>(st.sg, e, ciA, offA, nA, ciB, offB, nB, blk);
+    const int j = seg_entry<D, V, S>(st.sg, e, A, blk);
     V xj[KR * D];
-    ld_vec_n<KR * D, gather_l1<L_t, false>()>((const V*)L.x + (long long)j * KR * D, xj);
+    ld_vec_n<KR * D, true>((const V*)L.x + (long long)j * KR * D, xj);
 #pragma unroll
     for (int i = 0; i < KR; ++i)
 #pragma unroll
@@ -165,8 +152,8 @@ __device__ __forceinline__ void rowsm_pipelined(const LV<V>& L, int r0, int r1, 
 }
 
 // b_{l+1} = R r_l for coarse row I (one thread), every right-hand side.
-template <int D, int KR, typename V, typename L_t>
-__device__ __forceinline__ void restrictm_row(const L_t& L, int I) {
+template <int D, int KR, typename V>
+__device__ __forceinline__ void restrictm_row(const LV<V>& L, int I) {
   V acc[KR * D];
 #pragma unroll
   for (int q = 0; q < KR * D; ++q) acc[q] = V(0);
@@ -174,7 +161,7 @@ __device__ __forceinline__ void restrictm_row(const L_t& L, int I) {
     const int i = __ldg(L.rci + t);
     const V w = __ldg((const V*)L.rw + t);
     V ri[KR * D];
-    ld_vec_n<KR * D, gather_l1<L_t, false>()>((const V*)L.r + (long long)i * KR * D, ri);
+    ld_vec_n<KR * D, true>((const V*)L.r + (long long)i * KR * D, ri);
 #pragma unroll
     for (int q = 0; q < KR * D; ++q) acc[q] += w * ri[q];
   }
@@ -183,8 +170,8 @@ __device__ __forceinline__ void restrictm_row(const L_t& L, int I) {
 }
 
 // x_l += P x_{l+1} for fine row i (one thread), masked at dead dofs.
-template <int D, int KR, typename V, typename L_t>
-__device__ __forceinline__ void prolongm_row(const L_t& L, int i) {
+template <int D, int KR, typename V>
+__device__ __forceinline__ void prolongm_row(const LV<V>& L, int i) {
   V acc[KR * D];
 #pragma unroll
   for (int q = 0; q < KR * D; ++q) acc[q] = V(0);
@@ -192,7 +179,7 @@ __device__ __forceinline__ void prolongm_row(const L_t& L, int i) {
     const int J = __ldg(L.pci + t);
     const V w = __ldg((const V*)L.pw + t);
     V xJ[KR * D];
-    ld_vec_n<KR * D, gather_l1<L_t, false>()>((const V*)L.xc + (long long)J * KR * D, xJ);
+    ld_vec_n<KR * D, true>((const V*)L.xc + (long long)J * KR * D, xJ);
 #pragma unroll
     for (int q = 0; q < KR * D; ++q) acc[q] += w * xJ[q];
   }
@@ -547,11 +534,11 @@ __global__ void __launch_bounds__(tail_threads<D, float>(), 1)
   const TL<float>& L = A.lv[A.l0];
   const int n = L.nv * D, NT = nct * (int)blockDim.x;
   const int tid = (int)cluster_rank() * (int)blockDim.x + (int)threadIdx.x;
-  auto mix = [&](int t) { return ((long long)(t / D) * KR + i) * D + t % D; };
-  for (int t = tid; t < n; t += NT) __stcg(L.b + t, __ldcg(b + mix(t)));
+  auto at = [&](int t) { return ((long long)(t / D) * KR + i) * D + t % D; };
+  for (int t = tid; t < n; t += NT) __stcg(L.b + t, __ldcg(b + at(t)));
   cluster_sync_all();
   tail_run<D, float, S>(A);
-  for (int t = tid; t < n; t += NT) __stcg(x + mix(t), __ldcg((const float*)L.x + t));
+  for (int t = tid; t < n; t += NT) __stcg(x + at(t), __ldcg((const float*)L.x + t));
 }
 
 // ------------------------------------------------------------------ outer CG, KR right-hand sides (FP64)
